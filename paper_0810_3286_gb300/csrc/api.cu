@@ -132,7 +132,7 @@ struct svt_ctx {
   // Lanczos workspace
   double *Ub = nullptr, *Vb = nullptr;   // block bases (blocks of rows x b)
   double *T = nullptr, *S = nullptr, *theta = nullptr, *Xl = nullptr, *Wr = nullptr, *res = nullptr;
-  float* wsrc = nullptr;   // float32 leading Ritz vectors of the projected SVD (kKMax x kKMax)
+  double* psvd_ws = nullptr;              // workspace of the projected SVD
   double *G1 = nullptr, *G2 = nullptr, *G3 = nullptr, *gpart = nullptr, *R1 = nullptr, *dinv = nullptr;
   double *Rkeep = nullptr, *scale = nullptr;
   bool two_corrections = false;           // set once an orthonormality defect above 1e-6 was seen
@@ -626,21 +626,17 @@ static svt_status cycle_end(svt_ctx* c, int b, int J, int nk, bool copy_out) {
   // dimension b, so compact it first.
   CU(c, cudaMemcpy2DAsync(c->Rkeep, b * sizeof(double), c->S, kKMax * sizeof(double), b * sizeof(double), b,
                           cudaMemcpyDeviceToDevice, c->st));
-  // one-sided Jacobi stops when every column pair is orthogonal to 1e-11: Ritz vectors and values
-  // five orders beyond the float64 path's Lanczos tolerance (1e-6 sigma_1), and the float64
-  // kernel then finishes in one float64 sweep after its float32 preconditioning
+  // Ritz vectors and values five orders beyond the Lanczos tolerance (1e-6 sigma_1 for float64 values, 1e-4 for
+  // float32 and bfloat16 ones)
   const double tol_j = c->opt.lanczos_tol > 0 && c->opt.lanczos_tol < 1e-9
                            ? std::max(1e-15, 2.0 * K * 1.1102230246251565e-16)
-                           : 1e-11;
+                           : (c->prec == SVT_FP64 ? 1e-11 : 1e-9);
   // Ritz vectors formed in float64: the nk b that a thick restart of this shape keeps (they cover
   // every wanted triplet)
   const int nvec = std::max(1, nk) * b;
   l += prof_launch(c, SVT_PROF_JACOBI, 24.0 * K * K, [&] {
-    if (c->prec == SVT_FP64)
-      return launch_small_svd(c->T, kKMax, K, c->Rkeep, b, nvec, c->theta, c->Xl, c->Wr, c->res, tol_j, 60, c->err,
-                              c->dcount, c->st, c->opt.jacobi_cluster);
-    return launch_small_svd_mixed(c->T, kKMax, K, c->Rkeep, b, c->theta, c->Xl, c->Wr, c->res, nvec, c->wsrc, 2e-6,
-                                  60, c->err, c->dcount, c->st);
+    return launch_small_svd(c->T, kKMax, K, c->Rkeep, b, nvec, c->theta, c->Xl, c->Wr, c->res, tol_j, 60, c->err,
+                            c->dcount, c->psvd_ws, c->st, c->opt.jacobi_cluster);
   });
   TRY(launched(c, l));
   if (!copy_out) return SVT_OK;
@@ -1009,11 +1005,8 @@ static svt_status shrink_randomized(svt_ctx* c, double tau, int s_init, int* r_o
     TRY(orthonormalize(c, P, nullptr, 0, 0, n, l, nullptr, c->T, c->Vsh));
     const double tol_j = std::max(1e-15, 2.0 * l * 1.1102230246251565e-16);
     int lj = prof_launch(c, SVT_PROF_JACOBI, 24.0 * l * l, [&] {
-      if (c->prec == SVT_FP64)
-        return launch_small_svd(c->T, kKMax, l, nullptr, l, l, c->theta, c->Xl, c->Wr, c->res, tol_j, 60, c->err,
-                                c->dcount, c->st, c->opt.jacobi_cluster);
-      return launch_small_svd_mixed(c->T, kKMax, l, nullptr, l, c->theta, c->Xl, c->Wr, c->res, l, c->wsrc, 2e-6, 60,
-                                    c->err, c->dcount, c->st);
+      return launch_small_svd(c->T, kKMax, l, nullptr, l, l, c->theta, c->Xl, c->Wr, c->res, tol_j, 60, c->err,
+                              c->dcount, c->psvd_ws, c->st, c->opt.jacobi_cluster);
     });
     TRY(launched(c, lj));
     CU(c, cudaMemcpyAsync(c->h_pin, c->theta, sizeof(double) * l, cudaMemcpyDeviceToHost, c->st));
@@ -1274,7 +1267,7 @@ static svt_status create_body(svt_ctx* c, const int32_t* rows, const int32_t* co
   TRY(dalloc_t(c, &c->Xl, (size_t)kKMax * kKMax));
   TRY(dalloc_t(c, &c->Wr, (size_t)kKMax * kKMax));
   TRY(dalloc_t(c, &c->res, kKMax));
-  TRY(dalloc_t(c, &c->wsrc, (size_t)kKMax * kKMax));
+  TRY(dalloc_t(c, &c->psvd_ws, (size_t)psvd_workspace_doubles()));
   TRY(dalloc_t(c, &c->G1, kGramW * kBMax));
   TRY(dalloc_t(c, &c->G2, kGramW * kBMax));
   TRY(dalloc_t(c, &c->G3, kGramW * kBMax));
@@ -1337,7 +1330,7 @@ extern "C" size_t svt_estimate_device_bytes(int64_t m, int64_t n, int64_t nnz, c
   if (o.precision != SVT_FP64) b += 4 * (M + N) * kBMax + 4 * (M + N) * ((cap + 3) & ~3);
   b += 8 * (M + N) * (kKMax + kBMax);                        // Lanczos bases
   b += 8 * (3 * kKMax * kKMax + kKMax * kBMax + 3 * kGramW * kBMax + 3 * kBMax * kBMax + 256 + 4096);
-  b += 4 * kKMax * kKMax;                                    // float32 Ritz vectors of the projected SVD
+  b += 8 * (size_t)psvd_workspace_doubles();                 // projected SVD
   b += 8 * (size_t)gram_partial_doubles((int)std::max(m, n), kGramW / kBMax - 1, kBMax);
   // scratch of the structure build, peak (host inputs staged as int32, int32, float64)
   const size_t nmax = std::max(M, N) + 1;

@@ -130,15 +130,16 @@ int launch_orth_coop(double* P, const double* Q, long long q_stride, int nq, int
                      unsigned long long* counters, unsigned int* err, void* bar, int twoc, int max_grid,
                      cudaStream_t st, double repass, unsigned int spin_limit, int tc);
 
-// Jacobi SVD of the K x K matrix T (row-major, leading dimension ldT, block upper triangular with
-// b x b blocks, K <= 128): T = Xl diag(theta) Wr^T, theta decreasing; Xl, Wr written K x K
-// row-major (only the first nv columns of Wr are formed, the others are zero).  Also res[i] = || S (Xl rows [K-b, K), column i) ||
-// for the b x b block S (upper triangular, may be NULL -> res = 0).
-// counters[0] += 1, counters[1] += sweeps.
-// cluster: CTAs of the launch (0: a cluster of 8 where the device allows it, 1: one CTA).
+// Projected SVD (jacobi.cu) of the K x K matrix T (row-major, leading dimension ldT, block upper triangular with b x b
+// blocks, K <= 128 a multiple of 8): the leading nv triplets, theta decreasing; Xl, Wr K x K row-major.  The other
+// columns of Wr are zero, the other values approximate (their res INFINITY) or exact.  Also
+// res[i] = || S (Xl rows [K-b, K), column i) || for the b x b block S (upper triangular, may be NULL -> res = 0).
+// counters[0] += 1, counters[1] += sweeps and refinement steps.  ws: psvd_workspace_doubles() doubles.
+// cluster: CTAs of the launches (0: a cluster of 8 where the device allows it, 1: one CTA).  Two launches.
+long long psvd_workspace_doubles();
 int launch_small_svd(const double* T, int ldT, int K, const double* S, int b, int nv, double* theta, double* Xl,
                      double* Wr, double* res, double tol, int max_sweeps, unsigned int* err,
-                     unsigned long long* counters, cudaStream_t st, int cluster = 0);
+                     unsigned long long* counters, double* ws, cudaStream_t st, int cluster = 0);
 
 // Self-tests of the Newton helpers (out: 5 doubles per input): slots 0..3 rcp (2 steps, 1 step),
 // rsqrt (2 steps, 1 step) of jacobi.cu; slot 4 the pivot rsqrt of orth.cu.
@@ -172,13 +173,6 @@ int launch_cycle_decide(const LoopParams* prm, LoopState* st, const double* thet
 // Sets the dynamic shared-memory limits of the projected-SVD kernels (call before any stream
 // capture); returns 0 on success.
 int init_jacobi_attributes();
-
-// Float32-rotation Jacobi with float64 Ritz values for the leading nvec triplets (jacobi.cu); two
-// launches: the sweeps (one CTA), then the float64 refinement (nvec CTAs).  wsrc: nvec x K floats
-// of scratch.
-int launch_small_svd_mixed(const double* T, int ldT, int K, const double* S, int b, double* theta, double* Xl,
-                           double* Wr, double* res, int nvec, float* wsrc, double tol, int max_sweeps,
-                           unsigned int* err, unsigned long long* counters, cudaStream_t st);
 
 // Out (n x s) = sum over blocks i of B_i (n x b) W[i b .. i b + b, 0 .. s) , columns scaled by
 // scale[c] (or 1 when scale is NULL).  W: K x ldW row-major (K = nb * b).  OutF (may be NULL):
