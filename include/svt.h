@@ -130,12 +130,9 @@ typedef struct svt_options {
                              (the host finishes an iteration whose rank policy grows s_k); 0: the host
                              decides after every Lanczos cycle.  Not used with profiling
                              (svt_set_profile), use_graphs = 0 or the randomized engine. */
-  int orth_tf32;          /* coefficients of the first classical Gram-Schmidt pass of the cooperative
-                             orthonormalisation (C1 = Q^T P) from split-TF32 tensor-core products (about
-                             float32 accuracy); the projection, the second pass and a repeated pass are
-                             float64, so the basis stays orthonormal to float64 rounding.  0 (default): on
-                             for FP32 / BF16 values, off for FP64; 1: on; -1: off.  Needs orth_repass >= 0
-                             (off otherwise) */
+  int orth_tf32;          /* accepted and without effect: the coefficients of every Gram-Schmidt pass of the cooperative
+                             orthonormalisation have float64 accuracy at the speed the split-TF32 products
+                             this selected had */
   int jacobi_cluster;     /* projected SVD: 0 (default) a thread-block cluster of 8 CTAs where the device
                              allows it (the dense products, right vectors and residual estimates spread over
                              the cluster), else one CTA; 1: always one CTA (the same arithmetic but for the

@@ -137,7 +137,6 @@ struct svt_ctx {
   double *Rkeep = nullptr, *scale = nullptr;
   bool two_corrections = false;           // set once an orthonormality defect above 1e-6 was seen
   double orth_repass = 1e-6;              // defect above which a block's orthonormalisation pass is repeated
-  int orth_tc = 0;                        // first CGS pass's coefficients from split-TF32 tensor-core products
   unsigned int barrier_spins = kBarrierSpinLimit;
   int coop_grid = 0;                      // > 0: orthonormalise each block in one cooperative kernel
   void* gbar = nullptr;                   // its grid barrier (8 bytes, zeroed)
@@ -466,8 +465,7 @@ static svt_status orthonormalize(svt_ctx* c, double* P, const double* Q, long lo
     l += prof_launch_f(c, SVT_PROF_ORTH, bytes, flops, [&] {
       return launch_orth_coop(P, Q, q_stride, nq, rows, b, c->gpart, c->G1, c->G2, c->G3, Tcol, Tdiag, kKMax, Pf,
                               c->dcount, c->err, c->gbar, c->two_corrections ? 1 : 0, c->coop_grid, c->st,
-                              c->orth_repass, c->barrier_spins,
-                              c->orth_tc);
+                              c->orth_repass, c->barrier_spins);
     });
     if (l == 0) return fail(c, SVT_ERR_CUDA, "cooperative orthonormalisation launch failed: %s",
                             cudaGetErrorString(cudaGetLastError()));
@@ -748,7 +746,11 @@ static svt_status set_start_block(svt_ctx* c, int b, int warm) {
     CU(c, cudaMemcpy2DAsync(c->Vb, b * sizeof(double), c->Vwarm, c->warm_cols * sizeof(double), warm * sizeof(double),
                             n, cudaMemcpyDeviceToDevice, c->st));
   }
-  if (warm < b) l += launch_random_block(c->Vb, n, b, warm, next_seed(c), c->st);
+  // The residuals of converged Ritz vectors are rounding noise or nearly parallel, and the next block is made of them:
+  // 1e-9 of random directions (far below the tolerance; float32 products carry more noise than that) makes its columns
+  // independent.
+  const double eps = c->prec == SVT_FP64 && !(c->opt.lanczos_tol > 0 && c->opt.lanczos_tol < 1e-9) ? 1e-9 / std::sqrt((double)n) : 0.0;
+  if (warm < b || (warm > 0 && eps > 0.0)) l += launch_random_block(c->Vb, n, b, warm, next_seed(c), c->st, eps);
   return launched(c, l);
 }
 
@@ -1379,8 +1381,6 @@ extern "C" svt_status svt_create(int64_t m, int64_t n, int64_t nnz, const int32_
   c->vbytes = c->prec == SVT_FP64 ? 8 : 4;
   c->user_st = (cudaStream_t)o.stream;
   c->orth_repass = o.orth_repass == 0.0 ? 1e-6 : (o.orth_repass < 0.0 ? 0.0 : o.orth_repass);
-  // tensor-core first pass: by default for FP32 / BF16 values only; it needs the repeated pass
-  c->orth_tc = (o.orth_tf32 > 0 || (o.orth_tf32 == 0 && c->prec != SVT_FP64)) && c->orth_repass > 0.0 ? 1 : 0;
   svt_status s = SVT_OK;
   if (cudaGetDevice(&c->device) != cudaSuccess) {
     s = fail(c, SVT_ERR_CUDA, "no CUDA device");

@@ -65,20 +65,22 @@ int launch_basis_combine(const double* B, long long b_stride, int nb, int b, int
 // ------------------------------------------------------------------------------------------------
 // Random start columns: uniform(-1, 1) from SplitMix64 on the element index.
 // ------------------------------------------------------------------------------------------------
-__global__ void k_random_block(double* __restrict__ P, int n, int b, int c0, unsigned long long seed) {
+__global__ void k_random_block(double* __restrict__ P, int n, int b, int c0, unsigned long long seed,
+                               double eps) {
   long long total = (long long)n * b;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
     int c = (int)(e % b);
-    if (c < c0) continue;
-    P[e] = svt_uniform_pm1(seed, (unsigned long long)e);
+    const double u = svt_uniform_pm1(seed, (unsigned long long)e);
+    if (c >= c0) P[e] = u;
+    else if (eps > 0.0) P[e] += eps * u;
   }
 }
 
-int launch_random_block(double* P, int n, int b, int c0, uint64_t seed, cudaStream_t st) {
+int launch_random_block(double* P, int n, int b, int c0, uint64_t seed, cudaStream_t st, double eps) {
   long long total = (long long)n * b;
   int blocks = (int)svt_min_ll(svt_ceil_div(total, 256), 152LL * 8);
   if (blocks < 1) return 0;
-  k_random_block<<<blocks, 256, 0, st>>>(P, n, b, c0, seed);
+  k_random_block<<<blocks, 256, 0, st>>>(P, n, b, c0, seed, eps);
   return 1;
 }
 

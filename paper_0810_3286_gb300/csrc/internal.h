@@ -120,15 +120,14 @@ int launch_correct(const double* G3, const double* R1, double* Tdiag, int ldT, d
 // 8-byte barrier word (device).  Tcol / Tdiag / Pf may be NULL.  repass > 0: when the defect
 // max |P^T P - I| after the Cholesky pass exceeds it, the whole pass is repeated on its result and
 // the coefficients are composed (counters[4] += 1, counters[5] = max first-pass defect).
-// spin_limit: polls of a barrier wait before it gives up (SVT_DEVERR_BARRIER).  tc: the first
-// pass's coefficients C1 = Q^T P from TF32 tensor-core products (mma.sync), the rest float64.  Uses at most
+// spin_limit: polls of a barrier wait before it gives up (SVT_DEVERR_BARRIER).  Uses at most
 // min(orth_coop_init(), max_grid) CTAs and at most gram_partial_doubles(n, nq, b) partials.
 // Returns 1 when launched, 0 when the device cannot run it (the caller then uses the sequence).
 int orth_coop_init();
 int launch_orth_coop(double* P, const double* Q, long long q_stride, int nq, int n, int b, double* partial,
                      double* G1, double* G2, double* G3, double* Tcol, double* Tdiag, int ldT, float* Pf,
                      unsigned long long* counters, unsigned int* err, void* bar, int twoc, int max_grid,
-                     cudaStream_t st, double repass, unsigned int spin_limit, int tc);
+                     cudaStream_t st, double repass, unsigned int spin_limit);
 
 // Projected SVD (jacobi.cu) of the K x K matrix T (row-major, leading dimension ldT, block upper triangular with b x b
 // blocks, K <= 128 a multiple of 8): the leading nv triplets, theta decreasing; Xl, Wr K x K row-major.  The other
@@ -187,7 +186,7 @@ int launch_basis_combine(const double* B, long long b_stride, int nb, int b, int
 int launch_set_diagonal(double* T, int ldT, const double* d, int b, cudaStream_t st);
 
 // Fill an n x b block with uniform(-1, 1) numbers from SplitMix64 (columns c >= c0 only).
-int launch_random_block(double* P, int n, int b, int c0, uint64_t seed, cudaStream_t st);
+int launch_random_block(double* P, int n, int b, int c0, uint64_t seed, cudaStream_t st, double eps = 0.0);
 
 // Fused X-on-Omega + dual step + residual (precision 0: float64 values, 1: float32 values):
 //   x_p = sum_t Ut[i,t] V[j,t];  e = M_p - x_p;  y_out[p] = y_in[p] + delta e;
