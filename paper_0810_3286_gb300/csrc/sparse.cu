@@ -14,11 +14,13 @@ namespace svt {
 // SpMM over compressed segments: Out[s, :] = sum_{p in segment s} val[p] * X[idx[p], :].
 //
 // WPR warps share one segment (row of Y for Y V, column of Y for Y^T U using the column-major copy
-// of the values), each taking a contiguous slice of its entries, so that short products still
-// put enough warps on every SM to hide the gather latency.  Inside a warp a group of G lanes
+// of the values), each taking a contiguous slice of its entries, so that products of few segments still
+// put enough warps on every SM to hide the gather latency; with one warp a segment, a segment of over SPMM_LONG
+// entries is shared by the CTA's eight.  What bounds it: the float64 pipe (30000 segments of 120, b = 16: 178 -> 117 us,
+// 115 at the pipe's 0.50 T multiply-adds a second), L2 gathers in float32 (45.4 -> 37 us, 230 MB).  Inside a warp a group of G lanes
 // covers one sampled entry, each lane CPL adjacent columns of the b-wide dense row (one 16-byte
 // load of X: two float64 or four float32 columns); 32/G entries are in flight per step, four
-// steps are unrolled.  Lane partials are combined with xor shuffles and the WPR warp partials in
+// steps are unrolled.  Lane partials are combined by shuffles and the WPR warp partials in
 // shared memory, always in the same order (deterministic, no atomics).  Out is float64.
 //
 // The float32 path reads a float32 copy of the dense block and accumulates in float32: no
@@ -43,89 +45,151 @@ __device__ __forceinline__ void spmm_fma(AT (&acc)[CPL], AT v, const XT* __restr
   for (int q = 0; q < CPL; ++q) acc[q] = fmac(v, (AT)xcomp(x, q), acc[q]);
 }
 
+// A warp's sum over the entries [lo, hi) of one segment into w[0 .. n), the columns col .. col + n - 1 of the lanes with
+// n > 0.  Two sums a lane (shorter chains of additions; four need registers that cost resident warps: 30000 segments of 120,
+// b = 16, float32 37 -> 41 us); across the groups, a lane hands over half of its columns while it has several (fewer
+// shuffles and float64 adds than all columns on all lanes: float64 128 -> 117 us), and the last step is in float64.
+template <typename VT, typename XT, typename AT, int CPL>
+__device__ __forceinline__ void spmm_sum(const int32_t* __restrict__ idx, const VT* __restrict__ val,
+                                         const XT* __restrict__ X, int b, int G, int lo, int hi, double (&w)[CPL],
+                                         int& col, int& n) {
+  const int lane = threadIdx.x & 31;
+  const int ngrp = 32 / G;
+  const int c = CPL * (lane & (G - 1));
+  const bool active_col = c < b;
+  AT acc[2][CPL];
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) acc[k][q] = (AT)0;
+  int p = lo + lane / G;
+  for (; p + 3 * ngrp < hi; p += 4 * ngrp) {
+    int j[4];
+    AT v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      j[k] = __ldg(idx + p + k * ngrp);
+      v[k] = (AT)__ldg(val + p + k * ngrp);
+    }
+    if (active_col) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) spmm_fma<XT, AT, CPL>(acc[k & 1], v[k], X + (long long)j[k] * b + c);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (p + k * ngrp < hi) {
+      const int j = __ldg(idx + p + k * ngrp);
+      const AT v = (AT)__ldg(val + p + k * ngrp);
+      if (active_col) spmm_fma<XT, AT, CPL>(acc[k & 1], v, X + (long long)j * b + c);
+    }
+  }
+  AT s[CPL];
+#pragma unroll
+  for (int q = 0; q < CPL; ++q) s[q] = acc[0][q] + acc[1][q];
+  int o = G, off = 0;
+  n = CPL;
+  auto halve = [&](auto& x, int h) {               // of 2 h columns keep h
+    const bool up = lane & o;
+#pragma unroll
+    for (int q = 0; q < CPL / 2; ++q)
+      if (q < h) x[q] = (up ? x[q + h] : x[q]) + __shfl_xor_sync(0xffffffffu, up ? x[q] : x[q + h], o);
+    off += up ? h : 0;
+    n = h;
+    o <<= 1;
+  };
+  bool lead = active_col;
+  if (CPL == 4 && o < 16) halve(s, 2);
+  if (o < 16) halve(s, 1);
+  for (; o < 16; o <<= 1) {
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+    lead = lead && !(lane & o);
+  }
+#pragma unroll
+  for (int q = 0; q < CPL; ++q) w[q] = (double)s[q];
+  if (o == 16) {
+    if (n == 1) {
+      w[0] += __shfl_xor_sync(0xffffffffu, w[0], 16);
+      lead = lead && !(lane & 16);
+    } else if (n == 2) {
+      halve(w, 1);
+    } else {
+      halve(w, 2);
+    }
+  }
+  col = c + off;
+  if (!lead) n = 0;
+}
+
+// dst[0 .. n) = w, n = 0, 1, 2 or 4 (16-byte stores of pairs)
+template <int CPL>
+__device__ __forceinline__ void spmm_store(double* __restrict__ dst, const double (&w)[CPL], int n) {
+  if (n == 1) dst[0] = w[0];
+#pragma unroll
+  for (int q = 0; q < CPL; q += 2)
+    if (q + 2 <= n) *reinterpret_cast<double2*>(dst + q) = make_double2(w[q], w[q + 1]);
+}
+
+// Segments s0 + slot, slot = warp / WPR, by WPR > 1 warps each.  All threads of the CTA.
+template <typename VT, typename XT, typename AT>
+__device__ __forceinline__ void spmm_shared(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx,
+                                            const VT* __restrict__ val, const XT* __restrict__ X,
+                                            double* __restrict__ Out, int n_out, int b, int G, int WPR, int s0) {
+  constexpr int CPL = XRow<XT>::CPL;
+  __shared__ __align__(16) double part[SPMM_T / 32][64];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int slot = warp / WPR, wp = warp - slot * WPR;
+  const int s = s0 + slot;
+  if (s < n_out) {
+    const int a = ptr[s], e = ptr[s + 1];
+    const int chunk = (e - a + WPR - 1) / WPR;
+    const int lo = a + wp * chunk;
+    double w[CPL];
+    int col, n;
+    spmm_sum<VT, XT, AT, CPL>(idx, val, X, b, G, lo, min(e, lo + chunk), w, col, n);
+    spmm_store<CPL>(part[warp] + col, w, n);
+  }
+  __syncthreads();
+  if (wp == 0 && s < n_out) {
+    for (int c = lane; c < b; c += 32) {
+      double v = part[warp][c];
+      for (int k = 1; k < WPR; ++k) v += part[warp + k][c];
+      Out[(long long)s * b + c] = v;
+    }
+  }
+  __syncthreads();
+}
+
+// Segments longer than this are shared by the CTA's warps when a segment has one warp (WPR = 1): a warp takes ~0.7 us for 16
+// entries of 16 float64 columns.
+static constexpr int SPMM_LONG = 1024;
+
 // The segments s0 .. s0 + (SPMM_T / 32) / WPR - 1 of one product, by the whole CTA.
 template <typename VT, typename XT, typename AT>
 __device__ __forceinline__ void spmm_tile(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                                           const VT* __restrict__ val, const XT* __restrict__ X,
                                           double* __restrict__ Out, int n_out, int b, int G, int WPR, int s0) {
   constexpr int CPL = XRow<XT>::CPL;
-  __shared__ double part[SPMM_T / 32][64];
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const int slot = warp / WPR, wp = warp - slot * WPR;
-  const int gl = lane & (G - 1);
-  const int grp = lane / G;
-  const int ngrp = 32 / G;
-  const int c = CPL * gl;
-  const bool active_col = c < b;
-  {
-    const int s = s0 + slot;
-    AT acc[CPL];
-#pragma unroll
-    for (int q = 0; q < CPL; ++q) acc[q] = (AT)0;
-    if (s < n_out) {
-      const int a = ptr[s], e = ptr[s + 1];
-      const int len = e - a;
-      const int chunk = (len + WPR - 1) / WPR;
-      const int lo = a + wp * chunk;
-      const int hi = min(e, lo + chunk);
-      int p = lo + grp;
-      for (; p + 3 * ngrp < hi; p += 4 * ngrp) {
-        int j0 = __ldg(idx + p), j1 = __ldg(idx + p + ngrp), j2 = __ldg(idx + p + 2 * ngrp),
-            j3 = __ldg(idx + p + 3 * ngrp);
-        AT v0 = (AT)__ldg(val + p), v1 = (AT)__ldg(val + p + ngrp), v2 = (AT)__ldg(val + p + 2 * ngrp),
-           v3 = (AT)__ldg(val + p + 3 * ngrp);
-        if (active_col) {
-          spmm_fma<XT, AT, CPL>(acc, v0, X + (long long)j0 * b + c);
-          spmm_fma<XT, AT, CPL>(acc, v1, X + (long long)j1 * b + c);
-          spmm_fma<XT, AT, CPL>(acc, v2, X + (long long)j2 * b + c);
-          spmm_fma<XT, AT, CPL>(acc, v3, X + (long long)j3 * b + c);
-        }
-      }
-      for (; p < hi; p += ngrp) {
-        int j0 = __ldg(idx + p);
-        AT v0 = (AT)__ldg(val + p);
-        if (active_col) spmm_fma<XT, AT, CPL>(acc, v0, X + (long long)j0 * b + c);
-      }
+  if (WPR > 1) {
+    spmm_shared<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, WPR, s0);
+    return;
+  }
+  const int s = s0 + (threadIdx.x >> 5);
+  bool is_long = false;
+  if (s < n_out) {
+    const int a = ptr[s], e = ptr[s + 1];
+    is_long = e - a > SPMM_LONG;
+    if (!is_long) {
+      double w[CPL];
+      int col, n;
+      spmm_sum<VT, XT, AT, CPL>(idx, val, X, b, G, a, e, w, col, n);
+      spmm_store<CPL>(Out + (long long)s * b + col, w, n);
     }
-    for (int o = G; o < 32; o <<= 1) {
-#pragma unroll
-      for (int q = 0; q < CPL; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
-    }
-    if (WPR == 1) {
-      if (s < n_out && grp == 0 && active_col) {
-        double* dst = Out + (long long)s * b + c;
-#pragma unroll
-        for (int q = 0; q < CPL; q += 2) {
-          double2 w;
-          w.x = (double)acc[q]; w.y = (double)acc[q + 1];
-          *reinterpret_cast<double2*>(dst + q) = w;
-        }
-      }
-    } else {
-      if (grp == 0 && active_col) {
-#pragma unroll
-        for (int q = 0; q < CPL; ++q) part[warp][c + q] = (double)acc[q];
-      }
-      __syncthreads();
-      if (wp == 0 && s < n_out && grp == 0 && active_col) {
-        double w[CPL];
-#pragma unroll
-        for (int q = 0; q < CPL; ++q) w[q] = 0.0;
-        for (int k = 0; k < WPR; ++k) {
-#pragma unroll
-          for (int q = 0; q < CPL; ++q) w[q] += part[warp + k][c + q];
-        }
-        double* dst = Out + (long long)s * b + c;
-#pragma unroll
-        for (int q = 0; q < CPL; q += 2) {
-          double2 v2;
-          v2.x = w[q]; v2.y = w[q + 1];
-          *reinterpret_cast<double2*>(dst + q) = v2;
-        }
-      }
-      __syncthreads();
-    }
+  }
+  if (__syncthreads_or(is_long)) {
+    for (int k = s0; k < min(n_out, s0 + SPMM_T / 32); ++k)
+      if (ptr[k + 1] - ptr[k] > SPMM_LONG)
+        spmm_shared<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, SPMM_T / 32, k);
   }
 }
 
@@ -160,10 +224,14 @@ static void spmm_shape(int CPL, int b, long long nnz, int n_out, int wpr_overrid
   int G = 1;
   while (CPL * G < b) G <<= 1;   // G lanes x CPL columns >= b
   if (G > 32) G = 32;
-  // warps per segment from the mean segment length (entries per warp step = 32 / G)
+  // Warps per segment from the mean segment length (entries per warp step = 32 / G), up to 4096 warps in all: each warp of a
+  // split segment pays the adds of its shuffles, a barrier and a ragged last step, worth it only while the warps do not fill
+  // the machine (152 SMs with ~27 resident warps each).  Measured (us, b = 16, 1 / 2 / 4 warps a segment): 30000 segments of
+  // 120 float64 117 / 140 / 180, float32 37 / 50 / 80; 10000 of 120 float64 48 / 54 / 65; 2753 of 120 float64 23 / 22 / 25;
+  // 1000 of 120 float64 16.6 / 13.8 / 16.
   const double mean_len = nnz > 0 ? (double)nnz / n_out : 0.0;
   int WPR = 1;
-  while (WPR < 8 && mean_len / WPR > 8.0 * (32 / G)) WPR <<= 1;
+  while (WPR < 8 && mean_len / WPR > 8.0 * (32 / G) && (long long)n_out * WPR < 4096) WPR <<= 1;
   if (wpr_override == 1 || wpr_override == 2 || wpr_override == 4 || wpr_override == 8) WPR = wpr_override;
   *G_out = G;
   *WPR_out = WPR;
