@@ -457,8 +457,8 @@ svt_status svt_get_profile(svt_ctx* ctx, int64_t* launches, double* ms, double* 
  *   it to its square), [6] kernel launches, [7] shrinks whose Lanczos stagnated and were accepted
  *   at a relaxed tolerance (30x after 10 cycles, 300x after 25), [8] block orthonormalisations
  *   whose CGS2 + Cholesky QR pass was repeated (a defect above svt_options.orth_repass, or
- *   deflated columns replaced by fresh random directions), [9] largest defect of a first pass
- *   that was repeated for its defect, [10] SVT iterations run as one device-controlled graph
+ *   deflated columns, which keep their remainder plus a random direction at rounding level),
+ *   [9] largest defect of a first pass that was repeated for its defect, [10] SVT iterations run as one device-controlled graph
  *   (svt_options.device_loop).
  * Synchronises the stream.
  */
