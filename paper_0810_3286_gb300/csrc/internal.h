@@ -185,7 +185,8 @@ int launch_basis_combine(const double* B, long long b_stride, int nb, int b, int
 // T[i, i] = d[i] for i < b (row-major T, leading dimension ldT).
 int launch_set_diagonal(double* T, int ldT, const double* d, int b, cudaStream_t st);
 
-// Fill an n x b block with uniform(-1, 1) numbers from SplitMix64 (columns c >= c0 only).
+// Fill an n x b block with uniform(-1, 1) numbers from SplitMix64 (columns c >= c0 only); the columns before c0 get eps times
+// such numbers added.
 int launch_random_block(double* P, int n, int b, int c0, uint64_t seed, cudaStream_t st, double eps = 0.0);
 
 // Fused X-on-Omega + dual step + residual (precision 0: float64 values, 1: float32 values):
