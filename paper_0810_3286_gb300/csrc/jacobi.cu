@@ -208,7 +208,9 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_sweeps(PsvdArgs a) {
   __shared__ float s_diag[JMAXK];
   __shared__ int s_rank[JMAXK];
   __shared__ float s_new[2][JMAXK];      // diagonal after the rotations of a round: tops, then bottoms at 64
-  __shared__ int s_any[2], s_big[2];     // per rotation warp: a pair was rotated; at |cos| > sqrt(tol)
+  // Per rotation warp: a pair was rotated; at |cos| > sqrt(tol).  Two sets in turn: warps without blocks take no part in the
+  // rounds and may read a sweep's set while the rotation warps are already at the end of the next sweep.
+  __shared__ int s_any[2][2], s_big[2][2];
   __shared__ float s_dmax[2];
   constexpr int BW = PS_T / 32 - NP;     // block warps
   const int K = HC ? 2 * HC : a.K, h = K / 2;
@@ -447,8 +449,8 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_sweeps(PsvdArgs a) {
         big = __any_sync(0xffffffffu, big);
         const float m = warp_max(in ? fmaxf(dt, db) : 0.f);
         if (lane == 0) {
-          s_any[warp] = any;
-          s_big[warp] = big;
+          s_any[sweep & 1][warp] = any;
+          s_big[sweep & 1][warp] = big;
           s_dmax[warp] = m;
         }
       } else if (rounds) {
@@ -458,7 +460,9 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_sweeps(PsvdArgs a) {
       }
       __syncthreads();
       // quadratic convergence: a sweep whose pairs all had |cos| <= sqrt(tol) is followed by one more
-      const bool any = s_any[0] || (NP > 1 && s_any[1]), big = s_big[0] || (NP > 1 && s_big[1]);
+      const int* sa = s_any[sweep & 1];
+      const int* sb = s_big[sweep & 1];
+      const bool any = sa[0] || (NP > 1 && sa[1]), big = sb[0] || (NP > 1 && sb[1]);
       const bool stop = !any || final_sweep || sweep + 1 >= min(a.max_sweeps, 16);
       final_sweep = !big;
       if (tid == 0) __stcg(last_flag + (sweep & (PS_LOG - 1)), stop ? 1 : 0);
