@@ -122,6 +122,12 @@ __device__ __forceinline__ int next_place(int p, int h) {
   return i == 0 ? 2 : 2 * (i - 1) + 1;
 }
 
+// Integer that orders like x; NaNs come before or after all numbers.
+__device__ __forceinline__ int order_bits(float x) {
+  const int b = __float_as_int(x);
+  return b ^ ((b >> 31) & 0x7FFFFFFF);
+}
+
 __device__ __forceinline__ float rsqrt_ftz(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -499,12 +505,15 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_sweeps(PsvdArgs a) {
   for (int c = tid; c < K; c += PS_T) s_diag[c] = __ldcg(ws_diag + c);
   __syncthreads();
   for (int c = tid; c < K; c += PS_T) {
+    // by the bits (negative numbers reversed), equal ones by their index: a permutation, also with NaNs among them
     int r = 0;
-    const float d = s_diag[c];
-    for (int c2 = 0; c2 < K; ++c2) r += (s_diag[c2] > d || (s_diag[c2] == d && c2 < c)) ? 1 : 0;
-    // NaN entries compare false with everything: keep the ranks a permutation
-    s_rank[c] = isnan(d) ? c : r;
-    if (rank == 0) a.ws[PS_DIAG + (isnan(d) ? c : r)] = (double)d;
+    const int d = order_bits(s_diag[c]);
+    for (int c2 = 0; c2 < K; ++c2) {
+      const int d2 = order_bits(s_diag[c2]);
+      r += (d2 > d || (d2 == d && c2 < c)) ? 1 : 0;
+    }
+    s_rank[c] = r;
+    if (rank == 0) a.ws[PS_DIAG + r] = (double)s_diag[c];
   }
   __syncthreads();
   if (replays) {
@@ -689,9 +698,14 @@ __device__ __noinline__ void psvd_onesided(const PsvdArgs& a, double scale, doub
   }
   __syncthreads();
   for (int c = tid; c < K; c += PS_T) {
+    // by the bits of the magnitude, equal ones by their index: a permutation (order[] is an index), also with NaNs
     int r = 0;
-    for (int q = 0; q < K; ++q) r += (nrm[q] > nrm[c] || (nrm[q] == nrm[c] && q < c)) ? 1 : 0;
-    order[isnan(nrm[c]) ? c : r] = c;
+    const long long nc = __double_as_longlong(fabs(nrm[c]));
+    for (int q = 0; q < K; ++q) {
+      const long long nq = __double_as_longlong(fabs(nrm[q]));
+      r += (nq > nc || (nq == nc && q < c)) ? 1 : 0;
+    }
+    order[r] = c;
   }
   __syncthreads();
   for (int e = tid; e < K * K; e += PS_T) {
@@ -1146,9 +1160,9 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_refine(PsvdArgs a) {
   for (int i = tid; i < nv; i += PS_T) {
     // decreasing order (NaN bits order above everything, equal values by index: always a permutation)
     int r = 0;
-    const long long li = __double_as_longlong(s_lam[i]);
+    const long long li = __double_as_longlong(fabs(s_lam[i]));
     for (int q = 0; q < nv; ++q) {
-      const long long lq = __double_as_longlong(s_lam[q]);
+      const long long lq = __double_as_longlong(fabs(s_lam[q]));
       r += (lq > li || (lq == li && q < i)) ? 1 : 0;
     }
     s_rank[i] = r;
