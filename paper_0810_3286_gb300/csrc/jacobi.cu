@@ -691,9 +691,12 @@ __device__ __noinline__ void psvd_onesided(const PsvdArgs& a, double scale, doub
     for (int i = lane; i < K; i += 32) s2 = fma(sG[c * K + i], sG[c * K + i], s2);
     s2 = warp_sum(s2);
     if (lane == 0) {
-      const double th = s2 > 0.0 ? s2 * rsqrt_nr(s2, 2) : s2;
+      // Columns at the rounding of G hold no direction: x would repeat another one and T^T x / theta be of any size.  Their
+      // triplet is (0, 0, 0).
+      const bool null = s2 <= floor2;
+      const double th = null ? 0.0 : s2 * rsqrt_nr(s2, 2);
       nrm[c] = th;
-      rnrm[c] = th > 0.0 ? rcp_nr(th) : 0.0;
+      rnrm[c] = null ? 0.0 : rcp_nr(th);
     }
   }
   __syncthreads();
