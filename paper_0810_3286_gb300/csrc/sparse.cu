@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "internal.h"
@@ -130,23 +131,46 @@ __device__ __forceinline__ void spmm_store(double* __restrict__ dst, const doubl
     if (q + 2 <= n) *reinterpret_cast<double2*>(dst + q) = make_double2(w[q], w[q + 1]);
 }
 
+// A warp's sum over [lo, hi) like spmm_sum, in pieces of about `piece` entries (at least 2/3 of it, at most 3/2) whose sums
+// are added in float64: the chains of additions stay short however long the segment.  row: 64 doubles of the warp's own; a
+// lane keeps its columns there, no registers (nothing is kept of a single piece).
+template <typename VT, typename XT, typename AT, int CPL>
+__device__ __forceinline__ void spmm_pieces(const int32_t* __restrict__ idx, const VT* __restrict__ val,
+                                            const XT* __restrict__ X, int b, int G, int piece, int lo, int hi,
+                                            double* row, double (&w)[CPL], int& col, int& n) {
+  const int np = (hi - lo + piece / 2) / piece;
+  const int len = np > 1 ? (hi - lo + np - 1) / np : hi - lo;
+  for (int p = lo;;) {
+    const int q = min(hi, p + len);
+    spmm_sum<VT, XT, AT, CPL>(idx, val, X, b, G, p, q, w, col, n);
+    if (p > lo) {
+#pragma unroll
+      for (int k = 0; k < CPL; ++k)
+        if (k < n) w[k] += row[col + k];
+    }
+    p = q;
+    if (p >= hi) return;
+    spmm_store<CPL>(row + col, w, n);
+  }
+}
+
 // Segments s0 + slot, slot = warp / WPR, by WPR > 1 warps each.  All threads of the CTA.
 template <typename VT, typename XT, typename AT>
 __device__ __forceinline__ void spmm_shared(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                                             const VT* __restrict__ val, const XT* __restrict__ X,
-                                            double* __restrict__ Out, int n_out, int b, int G, int WPR, int s0) {
+                                            double* __restrict__ Out, int n_out, int b, int G, int WPR, int piece,
+                                            int s0, double (*part)[64]) {
   constexpr int CPL = XRow<XT>::CPL;
-  __shared__ __align__(16) double part[SPMM_T / 32][64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int slot = warp / WPR, wp = warp - slot * WPR;
   const int s = s0 + slot;
   if (s < n_out) {
     const int a = ptr[s], e = ptr[s + 1];
     const int chunk = (e - a + WPR - 1) / WPR;
-    const int lo = a + wp * chunk;
+    const int lo = min(e, a + wp * chunk);
     double w[CPL];
     int col, n;
-    spmm_sum<VT, XT, AT, CPL>(idx, val, X, b, G, lo, min(e, lo + chunk), w, col, n);
+    spmm_pieces<VT, XT, AT, CPL>(idx, val, X, b, G, piece, lo, min(e, lo + chunk), part[warp], w, col, n);
     spmm_store<CPL>(part[warp] + col, w, n);
   }
   __syncthreads();
@@ -168,10 +192,12 @@ static constexpr int SPMM_LONG = 1024;
 template <typename VT, typename XT, typename AT>
 __device__ __forceinline__ void spmm_tile(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                                           const VT* __restrict__ val, const XT* __restrict__ X,
-                                          double* __restrict__ Out, int n_out, int b, int G, int WPR, int s0) {
+                                          double* __restrict__ Out, int n_out, int b, int G, int WPR, int piece,
+                                          int s0) {
   constexpr int CPL = XRow<XT>::CPL;
+  __shared__ __align__(16) double part[SPMM_T / 32][64];
   if (WPR > 1) {
-    spmm_shared<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, WPR, s0);
+    spmm_shared<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, s0, part);
     return;
   }
   const int s = s0 + (threadIdx.x >> 5);
@@ -182,24 +208,24 @@ __device__ __forceinline__ void spmm_tile(const int32_t* __restrict__ ptr, const
     if (!is_long) {
       double w[CPL];
       int col, n;
-      spmm_sum<VT, XT, AT, CPL>(idx, val, X, b, G, a, e, w, col, n);
+      spmm_pieces<VT, XT, AT, CPL>(idx, val, X, b, G, piece, a, e, part[threadIdx.x >> 5], w, col, n);
       spmm_store<CPL>(Out + (long long)s * b + col, w, n);
     }
   }
   if (__syncthreads_or(is_long)) {
     for (int k = s0; k < min(n_out, s0 + SPMM_T / 32); ++k)
       if (ptr[k + 1] - ptr[k] > SPMM_LONG)
-        spmm_shared<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, SPMM_T / 32, k);
+        spmm_shared<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, SPMM_T / 32, piece, k, part);
   }
 }
 
 template <typename VT, typename XT, typename AT>
 __global__ void __launch_bounds__(SPMM_T)
 k_spmm(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx, const VT* __restrict__ val,
-       const XT* __restrict__ X, double* __restrict__ Out, int n_out, int b, int G, int WPR) {
+       const XT* __restrict__ X, double* __restrict__ Out, int n_out, int b, int G, int WPR, int piece) {
   const int segs_per_block = (SPMM_T / 32) / WPR;
   for (int s0 = blockIdx.x * segs_per_block; s0 < n_out; s0 += gridDim.x * segs_per_block)
-    spmm_tile<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, WPR, s0);
+    spmm_tile<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, s0);
 }
 
 // Ragged persistent form over a job list (batched engine): the tiles of all listed products form
@@ -214,13 +240,14 @@ __global__ void __launch_bounds__(SPMM_T) k_spmm_jobs(const __grid_constant__ Sp
     const SpmmJobDev& J = tab.job[k];
     const int segs_per_block = (SPMM_T / 32) / J.WPR;
     spmm_tile<VT, XT, AT>(J.ptr, J.idx, static_cast<const VT*>(J.val), static_cast<const XT*>(J.X), J.Out, J.n_out,
-                          J.b, J.G, J.WPR, (t - J.tile0) * segs_per_block);
+                          J.b, J.G, J.WPR, J.piece, (t - J.tile0) * segs_per_block);
   }
 }
 
-// Lanes per sampled entry (G) and warps per segment (WPR) of a product with b columns and mean
-// segment length nnz / n_out.  wpr_override > 0 replaces the rule (the batched engine's tuner).
-static void spmm_shape(int CPL, int b, long long nnz, int n_out, int wpr_override, int* G_out, int* WPR_out) {
+// Lanes per sampled entry (G), warps per segment (WPR) and entries of a piece of a product with b columns and mean
+// segment length nnz / n_out.  f32: float32 sums.  wpr_override > 0 replaces the rule for WPR (the batched engine's tuner).
+static void spmm_shape(int CPL, bool f32, int b, long long nnz, int n_out, int wpr_override, int* G_out, int* WPR_out,
+                       int* piece_out) {
   int G = 1;
   while (CPL * G < b) G <<= 1;   // G lanes x CPL columns >= b
   if (G > 32) G = 32;
@@ -233,19 +260,34 @@ static void spmm_shape(int CPL, int b, long long nnz, int n_out, int wpr_overrid
   int WPR = 1;
   while (WPR < 8 && mean_len / WPR > 8.0 * (32 / G) && (long long)n_out * WPR < 4096) WPR <<= 1;
   if (wpr_override == 1 || wpr_override == 2 || wpr_override == 4 || wpr_override == 8) WPR = wpr_override;
+  // Pieces: a lane's two sums take at most 16 entries each (times 3/2 where a length is no multiple of the piece), and no more
+  // than half of what `shares` warps would leave a lane of a mean segment.  In float64, with 2^-53 an addition, no more than
+  // all of that, and never less than half.  Measured, whole segments -> pieces (error of both products and the update against
+  // 64 bits, time of the three calls): 24000 x 20000, 520 entries a segment, b = 48: float32 2.9e-7 -> 8.7e-8, 3.33 -> 3.51 ms,
+  // float64 8.7e-16 -> 8.2e-16, 3.48 -> 3.53 ms; 9000 x 11000, 267, b = 32: float32 1.5e-7 -> 8.7e-8, 474 -> 507 us, float64 6.1e-16
+  // -> 5.8e-16, 477 -> 504 us.  Mean segments of 120 entries at b = 16 are one piece.
+  const int ngrp = 32 / G;
+  int shares = 1;
+  while (shares < 8 && mean_len / shares > 8.0 * ngrp) shares <<= 1;
+  int piece = 32 * ngrp;
+  if (shares > 1) {
+    const int half = 2 * (int)std::ceil(mean_len / shares);
+    piece = f32 ? std::min(piece, half) : std::max(std::min(piece, 2 * half), half);
+  }
   *G_out = G;
   *WPR_out = WPR;
+  *piece_out = piece;
 }
 
 template <typename VT, typename XT, typename AT>
 static void spmm_launch(const int32_t* ptr, const int32_t* idx, const VT* val, const XT* X, double* Out, int n_out,
                         int b, cudaStream_t st, long long nnz) {
   constexpr int CPL = XRow<XT>::CPL;
-  int G = 1, WPR = 1;
-  spmm_shape(CPL, b, nnz, n_out, 0, &G, &WPR);
+  int G = 1, WPR = 1, piece = 1;
+  spmm_shape(CPL, sizeof(AT) == 4, b, nnz, n_out, 0, &G, &WPR, &piece);
   const int segs_per_block = (SPMM_T / 32) / WPR;
   int blocks = (int)svt_min_ll(svt_ceil_div(n_out, segs_per_block), 152LL * 16);
-  k_spmm<VT, XT, AT><<<blocks, SPMM_T, 0, st>>>(ptr, idx, val, X, Out, n_out, b, G, WPR);
+  k_spmm<VT, XT, AT><<<blocks, SPMM_T, 0, st>>>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece);
 }
 
 // One launch for the products of a job list: precision as launch_spmm (0 float64, 1 float32 values
@@ -263,7 +305,7 @@ int launch_spmm_jobs(int precision, const SpmmJob* jobs, int n, int grid, cudaSt
     d.ptr = J.ptr; d.idx = J.idx; d.val = J.val; d.Out = J.Out; d.n_out = J.n_out; d.b = J.b;
     d.X = precision == 0 ? static_cast<const void*>(J.X) : static_cast<const void*>(J.Xf);
     if (!d.X) return 0;
-    spmm_shape(CPL, J.b, J.nnz, J.n_out, J.wpr, &d.G, &d.WPR);
+    spmm_shape(CPL, precision != 0, J.b, J.nnz, J.n_out, J.wpr, &d.G, &d.WPR, &d.piece);
     d.tile0 = tiles;
     tiles += (J.n_out + (SPMM_T / 32) / d.WPR - 1) / ((SPMM_T / 32) / d.WPR);
   }
