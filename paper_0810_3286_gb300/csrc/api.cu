@@ -633,8 +633,8 @@ static svt_status cycle_end(svt_ctx* c, int b, int J, int nk, bool copy_out) {
   // every wanted triplet)
   const int nvec = std::max(1, nk) * b;
   l += prof_launch(c, SVT_PROF_JACOBI, 24.0 * K * K, [&] {
-    return launch_small_svd(c->T, kKMax, K, c->Rkeep, b, nvec, c->theta, c->Xl, c->Wr, c->res, tol_j, 60, c->err,
-                            c->dcount, c->psvd_ws, c->st, c->opt.jacobi_cluster);
+    return launch_small_svd(c->T, kKMax, K, c->Rkeep, b, nvec, c->theta, c->Xl, c->Wr, c->res, tol_j,
+                            c->prec != SVT_FP64, 60, c->err, c->dcount, c->psvd_ws, c->st, c->opt.jacobi_cluster);
   });
   TRY(launched(c, l));
   if (!copy_out) return SVT_OK;
@@ -1007,8 +1007,8 @@ static svt_status shrink_randomized(svt_ctx* c, double tau, int s_init, int* r_o
     TRY(orthonormalize(c, P, nullptr, 0, 0, n, l, nullptr, c->T, c->Vsh));
     const double tol_j = std::max(1e-15, 2.0 * l * 1.1102230246251565e-16);
     int lj = prof_launch(c, SVT_PROF_JACOBI, 24.0 * l * l, [&] {
-      return launch_small_svd(c->T, kKMax, l, nullptr, l, l, c->theta, c->Xl, c->Wr, c->res, tol_j, 60, c->err,
-                              c->dcount, c->psvd_ws, c->st, c->opt.jacobi_cluster);
+      return launch_small_svd(c->T, kKMax, l, nullptr, l, l, c->theta, c->Xl, c->Wr, c->res, tol_j,
+                              c->prec != SVT_FP64, 60, c->err, c->dcount, c->psvd_ws, c->st, c->opt.jacobi_cluster);
     });
     TRY(launched(c, lj));
     CU(c, cudaMemcpyAsync(c->h_pin, c->theta, sizeof(double) * l, cudaMemcpyDeviceToHost, c->st));

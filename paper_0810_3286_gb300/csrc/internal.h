@@ -134,10 +134,12 @@ int launch_orth_coop(double* P, const double* Q, long long q_stride, int nq, int
 // columns of Wr are zero, the other values approximate (their res INFINITY) or exact.  Also
 // res[i] = || S (Xl rows [K-b, K), column i) || for the b x b block S (upper triangular, may be NULL -> res = 0).
 // counters[0] += 1, counters[1] += sweeps and refinement steps.  ws: psvd_workspace_doubles() doubles.
+// f32: T comes from float32 products; where the leading values span more than a factor 100, those below 2^-20 of the largest
+// (the products' rounding) are null, triplets (0, 0, 0).
 // cluster: CTAs of the launches (0: a cluster of 8 where the device allows it, 1: one CTA).  Two launches.
 long long psvd_workspace_doubles();
 int launch_small_svd(const double* T, int ldT, int K, const double* S, int b, int nv, double* theta, double* Xl,
-                     double* Wr, double* res, double tol, int max_sweeps, unsigned int* err,
+                     double* Wr, double* res, double tol, int f32, int max_sweeps, unsigned int* err,
                      unsigned long long* counters, double* ws, cudaStream_t st, int cluster = 0);
 
 // Self-tests of the Newton helpers (out: 5 doubles per input): slots 0..3 rcp (2 steps, 1 step),

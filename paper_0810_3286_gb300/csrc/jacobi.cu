@@ -19,9 +19,10 @@
 // 2e-12 .. 1.7e-11.  The sweeps are bound by the latency of a round (~310 cycles at K = 48: one barrier, two dependent
 // shared-memory reads, two reciprocal square roots), above K = 64 by instruction issue; the refinement by float64 latency
 // (64 cycles an operation) at K = 48 and by the float64 pipes of the cluster at K = 128.
-// A T whose leading nv values span more than a factor 100, or for which step 2 does not converge, is finished by
-// one-sided (Hestenes) Jacobi sweeps in float64 on G = T W in CTA 0, which are accurate relative to each singular
-// value (step 2's errors are relative to sigma_1^2).
+// A T whose leading nv values span more than a factor 100 has small values that the float32 M does not resolve: one-sided
+// (Hestenes) Jacobi sweeps in float32 on G = T W carry its rotations on.  In float64 contexts, and where step 2 does not
+// converge, T is then finished by one-sided sweeps in float64 in CTA 0, which are accurate relative to each singular value
+// (step 2's errors are relative to sigma_1^2).
 //
 // Residual estimates of the Lanczos relation: res_k = || S x_k[last b rows] || with S the b x b upper triangular
 // factor of the last block (Y^T U_J = V T^T + V_{J+1} S E_J^T).
@@ -104,6 +105,7 @@ struct PsvdArgs {
   int b, nv;
   double *theta, *Xl, *Wr, *res;
   double tol;
+  int f32;                    // T comes from float32 products
   int max_sweeps;
   unsigned int* err;
   unsigned long long* counters;
@@ -532,9 +534,24 @@ __device__ __forceinline__ long long max_bits(const double* v, int n) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// One-sided finish in float64
+// One-sided sweeps
 // ------------------------------------------------------------------------------------------------
-struct RotF64 {
+template <typename R>
+struct Rot;
+
+template <>
+struct Rot<float> {
+  static __device__ __forceinline__ void params(float al, float be, float ga, float& c, float& s, float& t) {
+    const float zeta = __fdividef(be - al, 2.f * ga), az = fabsf(zeta);
+    const float z2 = fmaf(zeta, zeta, 1.f);
+    t = copysignf(__fdividef(1.f, az + (az < 1e12f ? z2 * rsqrtf(z2) : az)), zeta);
+    c = rsqrtf(fmaf(t, t, 1.f));
+    s = c * t;
+  }
+};
+
+template <>
+struct Rot<double> {
   // One Newton step on each float32 seed (reciprocal y <- y (2 - x y), reciprocal square root
   // y <- y (3/2 - x y^2 / 2)): relative errors ~1e-14, so c^2 + s^2 = 1 to ~1e-14.
   static __device__ __forceinline__ void params(double al, double be, double ga, double& c, double& s, double& t) {
@@ -547,15 +564,13 @@ struct RotF64 {
   }
 };
 
-// Float64 sweeps of the one-sided Jacobi method on the columns of G (K x K, column-major in shared memory).  JL lanes per
-// column pair, JR = ceil(K / JL) rows each.  The squared column norms are formed in nrm2 at the start of a sweep and updated
-// by every rotation (al' = al - t ga, be' = be + t ga with t = s / c), so a pair needs one inner product.  Returns the
-// number of sweeps taken.
-static constexpr int JL = 8;
-
-template <int JR>
-__device__ __noinline__ int jacobi_sweeps(double* G, const unsigned char* sched, int K, double tol, int max_sweeps,
-                                          int* flag, double* nrm2, double floor2) {
+// Sweeps of the one-sided Jacobi method on the columns of G, in float32 on the columns of W too (both K x K, column-major
+// in shared memory).  JL lanes per column pair, JR >= ceil(K / JL) rows each.  The squared column norms are formed in nrm2 at
+// the start of a sweep and updated by every rotation (al' = al - t ga, be' = be + t ga with t = s / c), so a pair needs one
+// inner product.  Returns the number of sweeps taken.
+template <typename R, int JL, int JR>
+__device__ __noinline__ int jacobi_sweeps(R* G, R* W, const unsigned char* sched, int K, double tol, int max_sweeps,
+                                          int* flag, R* nrm2, R floor2) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int gl = lane & (JL - 1);                // lane inside the pair group
   const int gsub = lane / JL;                    // pair slot inside the warp
@@ -565,7 +580,7 @@ __device__ __noinline__ int jacobi_sweeps(double* G, const unsigned char* sched,
   for (; sweep < max_sweeps; ++sweep) {
     // the norms afresh: the updates below lose the small ones
     for (int c = warp; c < K; c += nw) {
-      double s2 = 0.0;
+      R s2 = 0;
       for (int i = lane; i < K; i += 32) s2 = fma(G[c * K + i], G[c * K + i], s2);
       s2 = warp_sum(s2);
       if (lane == 0) nrm2[c] = s2;
@@ -579,30 +594,31 @@ __device__ __noinline__ int jacobi_sweeps(double* G, const unsigned char* sched,
         const int pr = base + gsub;
         const bool has = pr < npairs;
         const int p = has ? rs[2 * pr] : 0, q = has ? rs[2 * pr + 1] : 0;
-        double* gp = G + p * K;
-        double* gq = G + q * K;
-        double a[JR], bq[JR];
-        double ga = 0;
+        R* gp = G + p * K;
+        R* gq = G + q * K;
+        R a[JR], bq[JR];
+        R ga = 0;
 #pragma unroll
         for (int k = 0; k < JR; ++k) {
           const int r = gl + JL * k;
           const bool in = has && r < K;
-          a[k] = in ? gp[r] : 0.0;
-          bq[k] = in ? gq[r] : 0.0;
+          a[k] = in ? gp[r] : (R)0;
+          bq[k] = in ? gq[r] : (R)0;
         }
         // read before the shuffles, written after them by one lane of the group
-        const double al = has ? nrm2[p] : 1.0, be = has ? nrm2[q] : 1.0;
+        const R al = has ? nrm2[p] : (R)1, be = has ? nrm2[q] : (R)1;
 #pragma unroll
         for (int k = 0; k < JR; ++k) ga += a[k] * bq[k];
 #pragma unroll
         for (int o = 1; o < JL; o <<= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-        // columns below 1e-13 of the largest are null: left alone
-        if (has && ga != 0.0 && al > floor2 && be > floor2) {
-          const double cs = fabs(ga) / (sqrt(al) * sqrt(be));
-          if (cs > tol) {
-            my_max = fmaxf(my_max, (float)cs);
-            double c, s, t;
-            RotF64::params(al, be, ga, c, s, t);
+        // null columns are left alone
+        if (has && ga != (R)0 && al > floor2 && be > floor2) {
+          // the cosine in float32 (it is only compared; a float64 division and two square roots take 2000 cycles)
+          const float cs = fabsf((float)ga) * rsqrtf((float)al) * rsqrtf((float)be);
+          if (cs > (float)tol) {
+            my_max = fmaxf(my_max, cs);
+            R c, s, t;
+            Rot<R>::params(al, be, ga, c, s, t);
             my_t = fmaxf(my_t, fabsf((float)t));
             if (gl == 0) {
               nrm2[p] = al - t * ga;
@@ -615,6 +631,19 @@ __device__ __noinline__ int jacobi_sweeps(double* G, const unsigned char* sched,
               if (r < K) {
                 gp[r] = c * a[k] - s * bq[k];
                 gq[r] = s * a[k] + c * bq[k];
+              }
+            }
+            if constexpr (sizeof(R) == 4) {
+              R* wp = W + p * K;
+              R* wq = W + q * K;
+#pragma unroll
+              for (int k = 0; k < JR; ++k) {
+                const int r = gl + JL * k;
+                if (r < K) {
+                  const R x = wp[r], y = wq[r];
+                  wp[r] = c * x - s * y;
+                  wq[r] = s * x + c * y;
+                }
               }
             }
           }
@@ -644,6 +673,10 @@ __device__ __noinline__ int jacobi_sweeps(double* G, const unsigned char* sched,
   return sweep + 1;
 }
 
+// Squared ratio to the largest value below which one is null: 1e-13, the rounding of G; 2^-20 where T holds the rounding of
+// float32 products.
+__device__ __forceinline__ double psvd_null2(const PsvdArgs& a) { return a.f32 ? 0x1p-40 : 1e-26; }
+
 // Round-robin tournament: in round r, pair 0 is (K-1, r) and pair i >= 1 is
 // ((r + i) mod (K-1), (r - i) mod (K-1)); every pair of columns meets once per sweep.
 __device__ void build_schedule(unsigned char* sched, int K) {
@@ -657,6 +690,50 @@ __device__ void build_schedule(unsigned char* sched, int K) {
     sched[2 * e] = (unsigned char)p;
     sched[2 * e + 1] = (unsigned char)q;
   }
+}
+
+// The leading values of a graded T span more than M = T^T T resolves in float32 (values below 6e-4 of the largest are mixed):
+// float32 one-sided sweeps on the columns of G = scale T W (workspace), which see 1e-7 of the largest, rotate W on.
+// Everything in CTA 0; the columns of W32 in decreasing order of their values, and their squares, back to the workspace.  smem:
+// K x K doubles; tmp as for psvd_onesided.
+__device__ __noinline__ void psvd_graded_sweeps(const PsvdArgs& a, float floor2, double* smem, double* tmp) {
+  __shared__ int flag;
+  const int K = a.K, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = PS_T / 32;
+  float* Wf = reinterpret_cast<float*>(a.ws + PS_WF);
+  float* sG = reinterpret_cast<float*>(smem);
+  float* sW = sG + K * K;
+  float* nrm = reinterpret_cast<float*>(tmp);
+  int* place = reinterpret_cast<int*>(nrm + K);
+  unsigned char* sched = reinterpret_cast<unsigned char*>(place + K);
+  build_schedule(sched, K);
+  for (int e = tid; e < K * K; e += PS_T) {
+    sG[e] = (float)__ldcg(a.ws + PS_G + e);
+    sW[e] = __ldcg(Wf + e);
+  }
+  __syncthreads();
+  const int sweeps = K <= 48 ? jacobi_sweeps<float, 16, 3>(sG, sW, sched, K, 2e-6, 16, &flag, nrm, floor2)
+                             : jacobi_sweeps<float, 8, 16>(sG, sW, sched, K, 2e-6, 16, &flag, nrm, floor2);
+  if (tid == 0 && a.counters) atomicAdd(&a.counters[1], (unsigned long long)sweeps);
+  __syncthreads();
+  for (int c = warp; c < K; c += nw) {
+    float s2 = 0.f;
+    for (int i = lane; i < K; i += 32) s2 = fmaf(sG[c * K + i], sG[c * K + i], s2);
+    s2 = warp_sum(s2);
+    if (lane == 0) nrm[c] = s2;
+  }
+  __syncthreads();
+  for (int c = tid; c < K; c += PS_T) {
+    int r = 0;
+    const int d = order_bits(nrm[c]);
+    for (int q = 0; q < K; ++q) {
+      const int dq = order_bits(nrm[q]);
+      r += (dq > d || (dq == d && q < c)) ? 1 : 0;
+    }
+    place[c] = r;
+    __stcg(a.ws + PS_DIAG + r, (double)nrm[c]);
+  }
+  __syncthreads();
+  for (int e = tid; e < K * K; e += PS_T) __stcg(Wf + place[e / K] * K + e % K, sW[e]);
 }
 
 // One-sided Jacobi finish in CTA 0: float64 sweeps on G = scale T W (workspace), tracked column norms, then
@@ -679,9 +756,9 @@ __device__ __noinline__ void psvd_onesided(const PsvdArgs& a, double scale, doub
     if (lane == 0) nrm[c] = s2;
   }
   __syncthreads();
-  const double floor2 = 1e-26 * __longlong_as_double(max_bits(nrm, K));
-  const int sweeps = K <= 48 ? jacobi_sweeps<6>(sG, sched, K, a.tol, a.max_sweeps, &flag, nrm, floor2)
-                             : jacobi_sweeps<16>(sG, sched, K, a.tol, a.max_sweeps, &flag, nrm, floor2);
+  const double floor2 = psvd_null2(a) * __longlong_as_double(max_bits(nrm, K));
+  const int sweeps = K <= 48 ? jacobi_sweeps<double, 8, 6>(sG, nullptr, sched, K, a.tol, a.max_sweeps, &flag, nrm, floor2)
+                             : jacobi_sweeps<double, 8, 16>(sG, nullptr, sched, K, a.tol, a.max_sweeps, &flag, nrm, floor2);
   if (tid == 0) {
     if (sweeps > a.max_sweeps) svt_set_error(a.err, SVT_DEVERR_JACOBI);
     if (a.counters) atomicAdd(&a.counters[1], (unsigned long long)sweeps);
@@ -691,8 +768,8 @@ __device__ __noinline__ void psvd_onesided(const PsvdArgs& a, double scale, doub
     for (int i = lane; i < K; i += 32) s2 = fma(sG[c * K + i], sG[c * K + i], s2);
     s2 = warp_sum(s2);
     if (lane == 0) {
-      // Columns at the rounding of G hold no direction: x would repeat another one and T^T x / theta be of any size.  Their
-      // triplet is (0, 0, 0).
+      // Null columns hold no direction: x would repeat another one and T^T x / theta be of any size.  Their triplet is
+      // (0, 0, 0).
       const bool null = s2 <= floor2;
       const double th = null ? 0.0 : s2 * rsqrt_nr(s2, 2);
       nrm[c] = th;
@@ -876,7 +953,7 @@ __device__ __noinline__ void psvd_start(const PsvdArgs& a, double* W0, int rank,
   float* sWf = reinterpret_cast<float*>(sA);
   float* sE = sWf + K * ld;
   float* sF = sE + K * ld;   // columns in hand, Kp apart
-  for (int e = tid; e < K * K; e += PS_T) sWf[(e / K) * ld + e % K] = Wf[e];
+  for (int e = tid; e < K * K; e += PS_T) sWf[(e / K) * ld + e % K] = __ldcg(Wf + e);
   __syncthreads();
   for (int t = rank * PS_T + tid; t < K / 2 * (K + 1); t += nct * PS_T) {
     int p, q;
@@ -960,6 +1037,49 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_refine(PsvdArgs a) {
   if (a.S)
     for (int e = tid; e < a.b * a.b; e += PS_T) sS[e] = a.S[e];
   psvd_start(a, W0, rank, nct, sA);
+  auto load_lambda = [&]() {
+    for (int i = tid; i < nv; i += PS_T) s_lam[i] = __ldcg(lam + i);
+    __syncthreads();
+  };
+  auto lambda_min = [&]() {   // NaN bits order above everything
+    long long m = __double_as_longlong(s_lam[0]);
+    for (int i = 1; i < nv; ++i) m = min(m, __double_as_longlong(s_lam[i]));
+    return __longlong_as_double(m);
+  };
+  // Leading values that span more than a factor 100 (the sweeps' diagonal is good to 1e-6 of its largest).  The rotations are
+  // carried on where the sweeps above have not resolved a cluster of small values; null values need none.  Then float64
+  // contexts and null values take the one-sided finish, float32 contexts a step of the refinement: cosines of 1e-6 or, for
+  // values below 3e-5 sigma_1, 1e-15 (sigma_1 / theta)^2.
+  // Measured (us a projected SVD, fully observed 300 x 300 rank 5 and 400 x 390 rank 30; the finish alone -> now): K = 48, noise
+  // 1e-3, float64 1660 -> 528, float32 1617 -> 238; K = 128, noise 1e-4, float64 7878 -> 2830, float32 8633 -> 1953; no noise
+  // (null values), float64 283 -> 187, float32 1504 -> 137.
+  double tol = a.tol;
+  if (__ldcg(a.ws + PS_DIAG + nv - 1) < 0.9e-4 * __ldcg(a.ws + PS_DIAG)) {
+    psvd_gz(a, Ts, ldT, W0, K, scale, false, rank, nct, sw, sg, part);
+    cl_sync();
+    load_lambda();
+    const double top = __longlong_as_double(max_bits(s_lam, nv)), floor2 = psvd_null2(a) * top;
+    bool null = false, some = false;   // null values; others that the sweeps may not have resolved
+    for (int i = 0; i < nv; ++i) {
+      null |= s_lam[i] <= floor2;
+      some |= s_lam[i] > floor2 && s_lam[i] < 1e-4 * top;
+    }
+    if (some) {
+      if (rank == 0) psvd_graded_sweeps(a, (float)floor2, sA, sw);
+      cl_sync();
+      psvd_start(a, W0, rank, nct, sA);
+      null = __ldcg(a.ws + PS_DIAG + nv - 1) <= floor2;
+      if (null || !a.f32) {
+        psvd_gz(a, Ts, ldT, W0, K, scale, false, rank, nct, sw, sg, part);
+        cl_sync();
+      }
+    }
+    if (null || !a.f32) {
+      if (rank == 0) psvd_onesided(a, scale, sA, sw);
+      return;
+    }
+    tol = fmax(tol, 1e-6);
+  }
   const double* Wtop = W0;   // where the final leading columns are
   bool converged = false;
   float th_prev = 0.f;
@@ -978,7 +1098,7 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_refine(PsvdArgs a) {
     // S, Theta: rows j = rank, rank + nct, ... of W, 16 at a time; four lanes per entry
     const int ldz = K + 4;
     for (int e = tid; e < nv * K; e += PS_T) sA[(e / K) * ldz + e % K] = __ldcg(a.ws + PS_Z + e);
-    for (int i = tid; i < K; i += PS_T) s_lam[i] = i < nv ? __ldcg(lam + i) : a.ws[PS_DIAG + i];
+    for (int i = tid; i < K; i += PS_T) s_lam[i] = i < nv ? __ldcg(lam + i) : __ldcg(a.ws + PS_DIAG + i);
     __syncthreads();
     // rounding of S, from the largest lambda (non-negative doubles compare like their bits)
     const float noise = 8.9e-16f * (float)__longlong_as_double(max_bits(s_lam, nv));
@@ -1044,7 +1164,7 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_refine(PsvdArgs a) {
       tsum += __ldcg(stat + 3 * q + 2);
     }
     th_prev = tmax;
-    if ((double)cmax <= a.tol) {   // the columns at hand are final
+    if ((double)cmax <= tol) {   // the columns at hand are final
       converged = true;
       break;
     }
@@ -1052,7 +1172,7 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_refine(PsvdArgs a) {
     // the one-sided sweeps do that (a single pair, |Theta|_F <= 1.11, stays here); so do NaNs, to be reported
     if (!(tsum <= 2.25f) || isinf(cmax)) break;
     // the step leaves errors of the size angle x cosine; the last step needs the leading columns only
-    const bool last = 4.0 * (double)tmax * (double)cmax <= a.tol && tmax < 5e-3f;
+    const bool last = 4.0 * (double)tmax * (double)cmax <= tol && tmax < 5e-3f;
     // W exp(Theta): the columns of Phi = Theta + Theta^2 / 2 + ..., as many powers as the angles ask for, in float32;
     // NC = 512 / Kp columns at a time, thread (t, j) entry j of column t.  The last step's W Phi (angles below 1e-5) is
     // added up in float32 as well, from float32 copies of W.
@@ -1148,11 +1268,8 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_refine(PsvdArgs a) {
   }
   if (rank == 0 && tid == 0 && a.counters) atomicAdd(&a.counters[1], (unsigned long long)it);
   cl_sync();
-  for (int i = tid; i < nv; i += PS_T) s_lam[i] = __ldcg(lam + i);
-  __syncthreads();
-  long long lmin = __double_as_longlong(s_lam[0]);
-  for (int i = 1; i < nv; ++i) lmin = min(lmin, __double_as_longlong(s_lam[i]));
-  if (!converged || __longlong_as_double(lmin) < 1e-4 * __longlong_as_double(max_bits(s_lam, nv))) {
+  load_lambda();
+  if (!converged || lambda_min() < (a.f32 ? psvd_null2(a) : 1e-4) * __longlong_as_double(max_bits(s_lam, nv))) {
     // one-sided sweeps on G = T W from the rotations of the float32 sweeps
     psvd_start(a, W0, rank, nct, sA);
     psvd_gz(a, Ts, ldT, W0, K, scale, false, rank, nct, sw, sg, part);
@@ -1201,7 +1318,7 @@ __global__ void __launch_bounds__(PS_T, 1) k_psvd_refine(PsvdArgs a) {
   }
   // the other triplets (not used by the rank policy, the restart or the shrink): values from the sweeps, no vectors
   for (int k = nv + rank * PS_T + tid; k < K; k += nct * PS_T) {
-    a.theta[k] = sqrt(fmax(a.ws[PS_DIAG + k], 0.0)) * unscale;
+    a.theta[k] = sqrt(fmax(__ldcg(a.ws + PS_DIAG + k), 0.0)) * unscale;
     a.res[k] = INFINITY;
   }
   for (int e = rank * PS_T + tid; e < K * (K - nv); e += nct * PS_T) {
@@ -1317,12 +1434,12 @@ static bool psvd_launch(Kernel* k, const PsvdArgs& a, int nct, size_t smem, cuda
 }
 
 int launch_small_svd(const double* T, int ldT, int K, const double* S, int b, int nv, double* theta, double* Xl,
-                     double* Wr, double* res, double tol, int max_sweeps, unsigned int* err,
+                     double* Wr, double* res, double tol, int f32, int max_sweeps, unsigned int* err,
                      unsigned long long* counters, double* ws, cudaStream_t st, int cluster) {
   // K is a multiple of the block size, itself a multiple of 8
   if (psvd_ctas() == 0 || K > JMAXK || K < 8 || (K & 7)) return 0;   // no launch; the caller's checks report it
   const int nct = cluster == 1 ? 1 : psvd_ctas();
-  const PsvdArgs a{T, ldT, K, S, b, nv < K ? nv : K, theta, Xl, Wr, res, tol, max_sweeps, err, counters, ws};
+  const PsvdArgs a{T, ldT, K, S, b, nv < K ? nv : K, theta, Xl, Wr, res, tol, f32, max_sweeps, err, counters, ws};
   if (!psvd_launch(psvd_sweeps_kernel(K), a, nct, psvd_sweeps_smem(K, nct), st)) return 0;
   return psvd_launch(k_psvd_refine, a, nct, psvd_refine_smem(K), st) ? 2 : 0;
 }
