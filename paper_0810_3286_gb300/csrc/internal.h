@@ -82,7 +82,7 @@ struct SpmmJobDev {
   const void* val;
   const void* X;
   double* Out;
-  int n_out, b, G, WPR, piece, tile0;
+  int n_out, b, G, WPR, piece, longw, tile0;
 };
 struct SpmmJobTable {
   int n, tiles;

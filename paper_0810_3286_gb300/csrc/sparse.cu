@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 
 #include "common.cuh"
@@ -16,8 +17,8 @@ namespace svt {
 //
 // WPR warps share one segment (row of Y for Y V, column of Y for Y^T U using the column-major copy
 // of the values), each taking a contiguous slice of its entries, so that products of few segments still
-// put enough warps on every SM to hide the gather latency; with one warp a segment, a segment of over SPMM_LONG
-// entries is shared by the CTA's eight.  What bounds it: the float64 pipe (30000 segments of 120, b = 16: 178 -> 117 us,
+// put enough warps on every SM to hide the gather latency; a segment that is much longer than the mean is shared by all
+// eight of a CTA.  What bounds it: the float64 pipe (30000 segments of 120, b = 16: 178 -> 117 us,
 // 115 at the pipe's 0.50 T multiply-adds a second), L2 gathers in float32 (45.4 -> 37 us, 230 MB).  Inside a warp a group of G lanes
 // covers one sampled entry, each lane CPL adjacent columns of the b-wide dense row (one 16-byte
 // load of X: two float64 or four float32 columns); 32/G entries are in flight per step, four
@@ -154,78 +155,67 @@ __device__ __forceinline__ void spmm_pieces(const int32_t* __restrict__ idx, con
   }
 }
 
-// Segments s0 + slot, slot = warp / WPR, by WPR > 1 warps each.  All threads of the CTA.
-template <typename VT, typename XT, typename AT>
-__device__ __forceinline__ void spmm_shared(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx,
-                                            const VT* __restrict__ val, const XT* __restrict__ X,
-                                            double* __restrict__ Out, int n_out, int b, int G, int WPR, int piece,
-                                            int s0, double (*part)[64]) {
-  constexpr int CPL = XRow<XT>::CPL;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int slot = warp / WPR, wp = warp - slot * WPR;
-  const int s = s0 + slot;
-  if (s < n_out) {
-    const int a = ptr[s], e = ptr[s + 1];
-    const int chunk = (e - a + WPR - 1) / WPR;
-    const int lo = min(e, a + wp * chunk);
-    double w[CPL];
-    int col, n;
-    spmm_pieces<VT, XT, AT, CPL>(idx, val, X, b, G, piece, lo, min(e, lo + chunk), part[warp], w, col, n);
-    spmm_store<CPL>(part[warp] + col, w, n);
-  }
-  __syncthreads();
-  if (wp == 0 && s < n_out) {
-    for (int c = lane; c < b; c += 32) {
-      double v = part[warp][c];
-      for (int k = 1; k < WPR; ++k) v += part[warp + k][c];
-      Out[(long long)s * b + c] = v;
-    }
-  }
-  __syncthreads();
-}
-
-// Segments longer than this are shared by the CTA's warps when a segment has one warp (WPR = 1): a warp takes ~0.7 us for 16
-// entries of 16 float64 columns.
-static constexpr int SPMM_LONG = 1024;
-
-// The segments s0 .. s0 + (SPMM_T / 32) / WPR - 1 of one product, by the whole CTA.
+// Tile `tile` of the `tiles` of one product, by the whole CTA: the segments tile + k tiles, k < (SPMM_T / 32) / WPR, WPR warps
+// each.  Segments of more than `longw` entries a warp are shared by all its warps; neighbours, which tend to be long together
+// (rows in the order of their popularity), belong to different tiles.  Measured (us, float64, b = 16): 10000 segments of 120 of
+// which the last eight have 1000, neighbours in one tile / in different ones: 110 / 57 (two segments a CTA with four warps
+// each: 73).
 template <typename VT, typename XT, typename AT>
 __device__ __forceinline__ void spmm_tile(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                                           const VT* __restrict__ val, const XT* __restrict__ X,
                                           double* __restrict__ Out, int n_out, int b, int G, int WPR, int piece,
-                                          int s0) {
-  constexpr int CPL = XRow<XT>::CPL;
-  __shared__ __align__(16) double part[SPMM_T / 32][64];
-  if (WPR > 1) {
-    spmm_shared<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, s0, part);
-    return;
-  }
-  const int s = s0 + (threadIdx.x >> 5);
+                                          int longw, int tile, int tiles) {
+  constexpr int CPL = XRow<XT>::CPL, NW = SPMM_T / 32;
+  __shared__ __align__(16) double part[NW][64];
+  const int warp = threadIdx.x >> 5;
+  // warp wp of the `share` warps of a segment [a, e): into Out where it is alone, else into part
+  auto sum = [&](int a, int e, int share, int wp, double* out) {
+    const int chunk = (e - a + share - 1) / share;
+    const int lo = min(e, a + wp * chunk);
+    double w[CPL];
+    int col, n;
+    spmm_pieces<VT, XT, AT, CPL>(idx, val, X, b, G, piece, lo, min(e, lo + chunk), part[warp], w, col, n);
+    spmm_store<CPL>((share > 1 ? part[warp] : out) + col, w, n);
+  };
+  // the sums of `share` warps from warp w0 on, by the threads t0, t0 + nt, ...
+  auto add = [&](int share, int w0, int t0, int nt, double* out) {
+    for (int c = t0; c < b; c += nt) {
+      double v = part[w0][c];
+      for (int k = 1; k < share; ++k) v += part[w0 + k][c];
+      out[c] = v;
+    }
+  };
+  const int slot = warp / WPR, wp = warp - slot * WPR, s = tile + slot * tiles;
+  const int limit = WPR < NW ? longw * WPR : INT_MAX;
   bool is_long = false;
   if (s < n_out) {
     const int a = ptr[s], e = ptr[s + 1];
-    is_long = e - a > SPMM_LONG;
-    if (!is_long) {
-      double w[CPL];
-      int col, n;
-      spmm_pieces<VT, XT, AT, CPL>(idx, val, X, b, G, piece, a, e, part[threadIdx.x >> 5], w, col, n);
-      spmm_store<CPL>(Out + (long long)s * b + col, w, n);
+    is_long = e - a > limit;
+    if (!is_long) sum(a, e, WPR, wp, Out + (long long)s * b);
+  }
+  const bool any = __syncthreads_or(is_long);
+  if (WPR > 1 && wp == 0 && s < n_out && !is_long) add(WPR, warp, threadIdx.x & 31, 32, Out + (long long)s * b);
+  if (any) {
+    for (int k = tile; k < n_out; k += tiles) {
+      const int a = ptr[k], e = ptr[k + 1];
+      if (e - a <= limit) continue;
+      __syncthreads();
+      sum(a, e, NW, warp, nullptr);
+      __syncthreads();
+      add(NW, 0, threadIdx.x, SPMM_T, Out + (long long)k * b);
     }
   }
-  if (__syncthreads_or(is_long)) {
-    for (int k = s0; k < min(n_out, s0 + SPMM_T / 32); ++k)
-      if (ptr[k + 1] - ptr[k] > SPMM_LONG)
-        spmm_shared<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, SPMM_T / 32, piece, k, part);
-  }
+  if (WPR > 1 || any) __syncthreads();
 }
 
 template <typename VT, typename XT, typename AT>
-__global__ void __launch_bounds__(SPMM_T)
+__global__ void __launch_bounds__(SPMM_T, 5)
 k_spmm(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx, const VT* __restrict__ val,
-       const XT* __restrict__ X, double* __restrict__ Out, int n_out, int b, int G, int WPR, int piece) {
+       const XT* __restrict__ X, double* __restrict__ Out, int n_out, int b, int G, int WPR, int piece, int longw) {
   const int segs_per_block = (SPMM_T / 32) / WPR;
-  for (int s0 = blockIdx.x * segs_per_block; s0 < n_out; s0 += gridDim.x * segs_per_block)
-    spmm_tile<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, s0);
+  const int tiles = (n_out + segs_per_block - 1) / segs_per_block;
+  for (int t = blockIdx.x; t < tiles; t += gridDim.x)
+    spmm_tile<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, longw, t, tiles);
 }
 
 // Ragged persistent form over a job list (batched engine): the tiles of all listed products form
@@ -240,14 +230,14 @@ __global__ void __launch_bounds__(SPMM_T) k_spmm_jobs(const __grid_constant__ Sp
     const SpmmJobDev& J = tab.job[k];
     const int segs_per_block = (SPMM_T / 32) / J.WPR;
     spmm_tile<VT, XT, AT>(J.ptr, J.idx, static_cast<const VT*>(J.val), static_cast<const XT*>(J.X), J.Out, J.n_out,
-                          J.b, J.G, J.WPR, J.piece, (t - J.tile0) * segs_per_block);
+                          J.b, J.G, J.WPR, J.piece, J.longw, t - J.tile0, (J.n_out + segs_per_block - 1) / segs_per_block);
   }
 }
 
 // Lanes per sampled entry (G), warps per segment (WPR) and entries of a piece of a product with b columns and mean
 // segment length nnz / n_out.  f32: float32 sums.  wpr_override > 0 replaces the rule for WPR (the batched engine's tuner).
 static void spmm_shape(int CPL, bool f32, int b, long long nnz, int n_out, int wpr_override, int* G_out, int* WPR_out,
-                       int* piece_out) {
+                       int* piece_out, int* longw_out) {
   int G = 1;
   while (CPL * G < b) G <<= 1;   // G lanes x CPL columns >= b
   if (G > 32) G = 32;
@@ -255,17 +245,21 @@ static void spmm_shape(int CPL, bool f32, int b, long long nnz, int n_out, int w
   // split segment pays the adds of its shuffles, a barrier and a ragged last step, worth it only while the warps do not fill
   // the machine (152 SMs with ~27 resident warps each).  Measured (us, b = 16, 1 / 2 / 4 warps a segment): 30000 segments of
   // 120 float64 117 / 140 / 180, float32 37 / 50 / 80; 10000 of 120 float64 48 / 54 / 65; 2753 of 120 float64 23 / 22 / 25;
-  // 1000 of 120 float64 16.6 / 13.8 / 16.
+  // 1000 of 120 float64 16.6 / 13.8 / 16.  Where a warp has over 48 steps to go, more and shorter ones even out the last wave
+  // and cost less, up to 16384 (limit of 4096 / 16384): 2797 segments of 348, b = 48, float64 113 / 109; 5000 of 300, b = 32, 105 /
+  // 89; 5000 of 250, b = 16, 51 / 47; 15000 of 300, b = 32, 253 / 242.
   const double mean_len = nnz > 0 ? (double)nnz / n_out : 0.0;
   int WPR = 1;
-  while (WPR < 8 && mean_len / WPR > 8.0 * (32 / G) && (long long)n_out * WPR < 4096) WPR <<= 1;
+  while (WPR < 8 && mean_len / WPR > 8.0 * (32 / G) &&
+         (long long)n_out * WPR < (mean_len / WPR > 48.0 * (32 / G) ? 16384 : 4096))
+    WPR <<= 1;
   if (wpr_override == 1 || wpr_override == 2 || wpr_override == 4 || wpr_override == 8) WPR = wpr_override;
   // Pieces: a lane's two sums take at most 16 entries each (times 3/2 where a length is no multiple of the piece), and no more
   // than half of what `shares` warps would leave a lane of a mean segment.  In float64, with 2^-53 an addition, no more than
   // all of that, and never less than half.  Measured, whole segments -> pieces (error of both products and the update against
-  // 64 bits, time of the three calls): 24000 x 20000, 520 entries a segment, b = 48: float32 2.9e-7 -> 8.7e-8, 3.33 -> 3.51 ms,
-  // float64 8.7e-16 -> 8.2e-16, 3.48 -> 3.53 ms; 9000 x 11000, 267, b = 32: float32 1.5e-7 -> 8.7e-8, 474 -> 507 us, float64 6.1e-16
-  // -> 5.8e-16, 477 -> 504 us.  Mean segments of 120 entries at b = 16 are one piece.
+  // 64 bits): 24000 x 20000, 520 entries a segment, b = 48: float32 2.9e-7 -> 8.7e-8 (the three calls 3.33 -> 3.51 ms), float64
+  // 8.7e-16 -> 8.2e-16 (3.48 -> 3.53 ms); 9000 x 11000, 267, b = 32: float32 1.5e-7 -> 8.8e-8, float64 6.1e-16 -> 5.8e-16.  Mean
+  // segments of 120 entries at b = 16 are one piece.
   const int ngrp = 32 / G;
   int shares = 1;
   while (shares < 8 && mean_len / shares > 8.0 * ngrp) shares <<= 1;
@@ -277,17 +271,20 @@ static void spmm_shape(int CPL, bool f32, int b, long long nnz, int n_out, int w
   *G_out = G;
   *WPR_out = WPR;
   *piece_out = piece;
+  // A warp takes three mean segments (or 64 steps) at most.  Measured (us, float64, b = 16, factors 8 / 4 / 3 / 2): 10000 segments
+  // of power-law lengths (exponent 2, mean 120) 96 / 84 / 79 / 79; 3000 of 120 with two of 1000 43 / 29 / 29 / 29.
+  *longw_out = std::max((int)std::min(3.0 * std::ceil(mean_len / WPR), 134217728.0), 64 * ngrp);
 }
 
 template <typename VT, typename XT, typename AT>
 static void spmm_launch(const int32_t* ptr, const int32_t* idx, const VT* val, const XT* X, double* Out, int n_out,
                         int b, cudaStream_t st, long long nnz) {
   constexpr int CPL = XRow<XT>::CPL;
-  int G = 1, WPR = 1, piece = 1;
-  spmm_shape(CPL, sizeof(AT) == 4, b, nnz, n_out, 0, &G, &WPR, &piece);
+  int G = 1, WPR = 1, piece = 1, longw = 1;
+  spmm_shape(CPL, sizeof(AT) == 4, b, nnz, n_out, 0, &G, &WPR, &piece, &longw);
   const int segs_per_block = (SPMM_T / 32) / WPR;
   int blocks = (int)svt_min_ll(svt_ceil_div(n_out, segs_per_block), 152LL * 16);
-  k_spmm<VT, XT, AT><<<blocks, SPMM_T, 0, st>>>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece);
+  k_spmm<VT, XT, AT><<<blocks, SPMM_T, 0, st>>>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, longw);
 }
 
 // One launch for the products of a job list: precision as launch_spmm (0 float64, 1 float32 values
@@ -305,7 +302,7 @@ int launch_spmm_jobs(int precision, const SpmmJob* jobs, int n, int grid, cudaSt
     d.ptr = J.ptr; d.idx = J.idx; d.val = J.val; d.Out = J.Out; d.n_out = J.n_out; d.b = J.b;
     d.X = precision == 0 ? static_cast<const void*>(J.X) : static_cast<const void*>(J.Xf);
     if (!d.X) return 0;
-    spmm_shape(CPL, precision != 0, J.b, J.nnz, J.n_out, J.wpr, &d.G, &d.WPR, &d.piece);
+    spmm_shape(CPL, precision != 0, J.b, J.nnz, J.n_out, J.wpr, &d.G, &d.WPR, &d.piece, &d.longw);
     d.tile0 = tiles;
     tiles += (J.n_out + (SPMM_T / 32) / d.WPR - 1) / ((SPMM_T / 32) / d.WPR);
   }
