@@ -1005,7 +1005,8 @@ static svt_status shrink_randomized(svt_ctx* c, double tau, int s_init, int* r_o
     TRY(prod(true, Q, c->Ush, P));
     CU(c, cudaMemsetAsync(c->T, 0, sizeof(double) * kKMax * kKMax, c->st));
     TRY(orthonormalize(c, P, nullptr, 0, 0, n, l, nullptr, c->T, c->Vsh));
-    const double tol_j = std::max(1e-15, 2.0 * l * 1.1102230246251565e-16);
+    // (float32 products: as in a Lanczos cycle)
+    const double tol_j = c->prec == SVT_FP64 ? std::max(1e-15, 2.0 * l * 1.1102230246251565e-16) : 1e-9;
     int lj = prof_launch(c, SVT_PROF_JACOBI, 24.0 * l * l, [&] {
       return launch_small_svd(c->T, kKMax, l, nullptr, l, l, c->theta, c->Xl, c->Wr, c->res, tol_j,
                               c->prec != SVT_FP64, 60, c->err, c->dcount, c->psvd_ws, c->st, c->opt.jacobi_cluster);
