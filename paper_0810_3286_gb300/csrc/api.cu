@@ -132,7 +132,6 @@ struct svt_ctx {
   // Lanczos workspace
   double *Ub = nullptr, *Vb = nullptr;   // block bases (blocks of rows x b)
   double *T = nullptr, *S = nullptr, *theta = nullptr, *Xl = nullptr, *Wr = nullptr, *res = nullptr;
-  double* psvd_ws = nullptr;              // workspace of the projected SVD
   double *G1 = nullptr, *G2 = nullptr, *G3 = nullptr, *gpart = nullptr, *R1 = nullptr, *dinv = nullptr;
   double *Rkeep = nullptr, *scale = nullptr;
   bool two_corrections = false;           // set once an orthonormality defect above 1e-6 was seen
@@ -634,7 +633,7 @@ static svt_status cycle_end(svt_ctx* c, int b, int J, int nk, bool copy_out) {
   const int nvec = std::max(1, nk) * b;
   l += prof_launch(c, SVT_PROF_JACOBI, 24.0 * K * K, [&] {
     return launch_small_svd(c->T, kKMax, K, c->Rkeep, b, nvec, c->theta, c->Xl, c->Wr, c->res, tol_j,
-                            c->prec != SVT_FP64, 60, c->err, c->dcount, c->psvd_ws, c->st, c->opt.jacobi_cluster);
+                            c->prec != SVT_FP64, 60, c->err, c->dcount, c->gpart, c->st, c->opt.jacobi_cluster);
   });
   TRY(launched(c, l));
   if (!copy_out) return SVT_OK;
@@ -1009,7 +1008,7 @@ static svt_status shrink_randomized(svt_ctx* c, double tau, int s_init, int* r_o
     const double tol_j = c->prec == SVT_FP64 ? std::max(1e-15, 2.0 * l * 1.1102230246251565e-16) : 1e-9;
     int lj = prof_launch(c, SVT_PROF_JACOBI, 24.0 * l * l, [&] {
       return launch_small_svd(c->T, kKMax, l, nullptr, l, l, c->theta, c->Xl, c->Wr, c->res, tol_j,
-                              c->prec != SVT_FP64, 60, c->err, c->dcount, c->psvd_ws, c->st, c->opt.jacobi_cluster);
+                              c->prec != SVT_FP64, 60, c->err, c->dcount, c->gpart, c->st, c->opt.jacobi_cluster);
     });
     TRY(launched(c, lj));
     CU(c, cudaMemcpyAsync(c->h_pin, c->theta, sizeof(double) * l, cudaMemcpyDeviceToHost, c->st));
@@ -1224,6 +1223,12 @@ static svt_status build_structure(svt_ctx* c, const int32_t* rows_d, const int32
   return SVT_OK;
 }
 
+// Scratch of the orthonormalisation (partial Grams: (nq + 1) b <= kGramW columns against b <= 32, at most kGramW x 32 entries
+// per row chunk) and of the projected SVD, which follow each other on the context's stream.
+static size_t scratch_doubles(int64_t m, int64_t n) {
+  return (size_t)std::max(gram_partial_doubles((int)std::max(m, n), kGramW / kBMax - 1, kBMax), psvd_workspace_doubles());
+}
+
 // Allocations, input staging and the Omega storage build of svt_create.  Local temporaries are
 // released when this returns, before svt_create destroys a failed context.
 static svt_status create_body(svt_ctx* c, const int32_t* rows, const int32_t* cols, const double* M_omega) {
@@ -1270,7 +1275,6 @@ static svt_status create_body(svt_ctx* c, const int32_t* rows, const int32_t* co
   TRY(dalloc_t(c, &c->Xl, (size_t)kKMax * kKMax));
   TRY(dalloc_t(c, &c->Wr, (size_t)kKMax * kKMax));
   TRY(dalloc_t(c, &c->res, kKMax));
-  TRY(dalloc_t(c, &c->psvd_ws, (size_t)psvd_workspace_doubles()));
   TRY(dalloc_t(c, &c->G1, kGramW * kBMax));
   TRY(dalloc_t(c, &c->G2, kGramW * kBMax));
   TRY(dalloc_t(c, &c->G3, kGramW * kBMax));
@@ -1281,8 +1285,7 @@ static svt_status create_body(svt_ctx* c, const int32_t* rows, const int32_t* co
   TRY(dalloc(c, &c->gbar, 8));
   CU(c, cudaMemsetAsync(c->gbar, 0, 8, c->st));
   CU(c, cudaMemsetAsync(c->dcount, 0, 8 * sizeof(unsigned long long), c->st));
-  // (nq + 1) b <= kGramW columns against b <= 32: at most kGramW x 32 entries per row chunk
-  TRY(dalloc_t(c, &c->gpart, (size_t)gram_partial_doubles((int)std::max(m, n), kGramW / kBMax - 1, kBMax)));
+  TRY(dalloc_t(c, &c->gpart, scratch_doubles(m, n)));
   TRY(dalloc_t(c, &c->Rkeep, kBMax * kBMax));
   TRY(dalloc_t(c, &c->scale, kKMax));
   TRY(dalloc_t(c, &c->dl_prm, 1));
@@ -1333,8 +1336,7 @@ extern "C" size_t svt_estimate_device_bytes(int64_t m, int64_t n, int64_t nnz, c
   if (o.precision != SVT_FP64) b += 4 * (M + N) * kBMax + 4 * (M + N) * ((cap + 3) & ~3);
   b += 8 * (M + N) * (kKMax + kBMax);                        // Lanczos bases
   b += 8 * (3 * kKMax * kKMax + kKMax * kBMax + 3 * kGramW * kBMax + 3 * kBMax * kBMax + 256 + 4096);
-  b += 8 * (size_t)psvd_workspace_doubles();                 // projected SVD
-  b += 8 * (size_t)gram_partial_doubles((int)std::max(m, n), kGramW / kBMax - 1, kBMax);
+  b += 8 * scratch_doubles(m, n);                            // partial Grams, projected SVD
   // scratch of the structure build, peak (host inputs staged as int32, int32, float64)
   const size_t nmax = std::max(M, N) + 1;
   size_t pow2 = 1;

@@ -121,7 +121,7 @@ int launch_correct(const double* G3, const double* R1, double* Tdiag, int ldT, d
 // max |P^T P - I| after the Cholesky pass exceeds it, the whole pass is repeated on its result and
 // the coefficients are composed (counters[4] += 1, counters[5] = max first-pass defect).
 // spin_limit: polls of a barrier wait before it gives up (SVT_DEVERR_BARRIER).  Uses at most
-// min(orth_coop_init(), max_grid) CTAs and at most gram_partial_doubles(n, nq, b) partials.
+// min(orth_coop_init(), max_grid) CTAs and at most gram_partial_doubles(n, 4, 32) partials ((nq + 1) b <= 160).
 // Returns 1 when launched, 0 when the device cannot run it (the caller then uses the sequence).
 int orth_coop_init();
 int launch_orth_coop(double* P, const double* Q, long long q_stride, int nq, int n, int b, double* partial,

@@ -60,11 +60,14 @@ static int gram_rows_per_cta(int n) {
 }
 
 // Upper bound on the row chunks of any launch with n' <= n rows: each chunk has >= GRAM_SUB rows
-// and >= ceil(n' / 304) rows, so there are at most min(ceil(n / GRAM_SUB), 304) chunks.
+// and >= ceil(n' / 304) rows, so there are at most min(ceil(n / GRAM_SUB), 304) chunks.  k_orth_coop on a small grid
+// alternates between two sets, of chunks of 16 rows (of 8 only for 8 columns, whose Grams are a fifth of the largest).
+static constexpr int OC_SETS_GRID = 32;   // largest grid with two sets
 long long gram_partial_doubles(int n, int nq, int b) {
-  long long nblk = (n + GRAM_SUB - 1) / GRAM_SUB;
-  if (nblk > 2 * 152) nblk = 2 * 152;
-  return 2 * nblk * (long long)(nq + 1) * b * b;   // k_orth_coop alternates between two sets
+  const long long rows = n;
+  const long long nblk = std::max(std::min((rows + GRAM_SUB - 1) / GRAM_SUB, 2LL * 152),
+                                  2 * std::min((rows + 15) / 16, (long long)OC_SETS_GRID));
+  return nblk * (nq + 1) * b * b;
 }
 
 // Entry layout of a Gram G = [Q_0 .. Q_{nq-1}, P]^T P: the nq b x b blocks Q_k^T P row-major,
@@ -1088,7 +1091,7 @@ struct OrthCoopArgs {
   int nq, n, g, rpc;          // rpc: rows per CTA
   int fma;                    // float64 instructions instead of digit products (b = 8, small n)
   double *partial, *G1, *G2, *G3;
-  long long part_half;        // doubles of one of the two sets of partials
+  long long part_half;        // doubles of one of the two sets of partials (0: one set)
   double *Tcol, *Tdiag;       // coefficient outputs (may be NULL), leading dimension ldT
   int ldT;
   float* Pf;                  // float32 copy of the result (may be NULL)
@@ -1187,7 +1190,8 @@ __global__ void __launch_bounds__(ORTH_T, 2) k_orth_coop(OrthCoopArgs a) {
     }
     dg_update<B>(a.Q, a.q_stride, a.nq, sC, s_ec, eq, a.P, r0, r1, s_mp[cur], w0, nw - w0, s_red, bar);
   };
-  // Two sets of partials in turn: a CTA may still read one Gram's while another writes the next one's.
+  // Where every CTA adds up a Gram for itself, one may still read its partials while another writes the next Gram's: two sets
+  // in turn.  (Else a barrier follows the sums, and the sets are the same.)
   double* partial = a.partial;
   // After a partial Gram: the sums of all CTAs, the coefficients in sC and the rest in sTail.  false: a barrier gave up.
   auto gram_sums = [&](int nq, bool first, double* G, const double* Gprev, double* Tcol, double* sTail,
@@ -1196,7 +1200,7 @@ __global__ void __launch_bounds__(ORTH_T, 2) k_orth_coop(OrthCoopArgs a) {
     if (!svt_grid_barrier(a.bar, a.err, a.spin_limit)) return false;
     const double* part = partial;
     partial = partial == a.partial ? a.partial + a.part_half : a.partial;
-    if (nq == 0 && nb <= 32) {   // (with coefficients the CTAs' reads take longer than the barrier: 16000 cycles at n = 1000)
+    if (nq == 0 && nb <= OC_SETS_GRID) {   // (with coefficients the CTAs' reads take longer than the barrier: 16000 cycles at n = 1000)
       reduce_all(part, nb, E, G, Gprev, Tcol, a.ldT, nc, B, sC, sTail, err);
     } else {
       reduce_entries(part, nb, E, G, Gprev, Tcol, a.ldT, nc, B, err);
@@ -1424,7 +1428,7 @@ int launch_orth_coop(double* P, const double* Q, long long q_stride, int nq, int
   const int grid = (n + rpc - 1) / rpc;
   OrthCoopArgs a;
   a.P = P; a.Q = Q; a.q_stride = q_stride; a.nq = nq; a.n = n; a.g = row_group(b); a.rpc = rpc; a.fma = fma ? 1 : 0;
-  a.partial = partial; a.part_half = (long long)grid * gram_entries(nq, b, false); a.G1 = G1; a.G2 = G2; a.G3 = G3;
+  a.partial = partial; a.part_half = grid <= OC_SETS_GRID ? (long long)grid * gram_entries(nq, b, false) : 0; a.G1 = G1; a.G2 = G2; a.G3 = G3;
   a.Tcol = Tcol; a.Tdiag = Tdiag; a.ldT = ldT; a.Pf = Pf;
   a.counters = counters; a.err = err; a.bar = static_cast<unsigned int*>(bar); a.twoc = twoc;
   a.repass = repass;
