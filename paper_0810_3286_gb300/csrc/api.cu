@@ -745,9 +745,11 @@ static svt_status set_start_block(svt_ctx* c, int b, int warm) {
     CU(c, cudaMemcpy2DAsync(c->Vb, b * sizeof(double), c->Vwarm, c->warm_cols * sizeof(double), warm * sizeof(double),
                             n, cudaMemcpyDeviceToDevice, c->st));
   }
-  // The residuals of converged Ritz vectors are rounding noise or nearly parallel, and the next block is made of them:
-  // 1e-9 of random directions (far below the tolerance; float32 products carry more noise than that) makes its columns
-  // independent.
+  // The residuals of converged Ritz vectors are rounding noise or nearly parallel, and the next block is made of them: 1e-9
+  // of random directions (float32 products carry more noise than that) makes its columns independent.  That is up to 0.6 of
+  // the tolerance, and no tolerance needs another cycle for it: three solves each of 200 x 200 and 1000 x 1000 at 1e-9 take
+  // 1252 and 1168 cycles with it as with a thousandth of it, which leaves 2 and 13 blocks to a repeated pass (with it none).
+  // Tighter tolerances do without it and repeat the pass (18 blocks of 1000 x 1000).
   const double eps = c->prec == SVT_FP64 && !(c->opt.lanczos_tol > 0 && c->opt.lanczos_tol < 1e-9) ? 1e-9 / std::sqrt((double)n) : 0.0;
   if (warm < b || (warm > 0 && eps > 0.0)) l += launch_random_block(c->Vb, n, b, warm, next_seed(c), c->st, eps);
   return launched(c, l);

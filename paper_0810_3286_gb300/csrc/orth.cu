@@ -573,7 +573,10 @@ __device__ void correct_rows(const double* __restrict__ sU, double* __restrict__
   }
 }
 
-// The same with the correction P U formed in float32, for |U| <= 1e-9: its rounding is below that of P.  sUf: U in float32.
+// The same with the correction P U formed in float32, for |U| <= kCorrectF32: the two conversions and up to b / 2 + 1 roundings
+// of each of its b terms are at most b (b / 2 + 3) 2^-24 |U| of the row's largest element, below 2^-53 of it for b = 32.  sUf: U
+// in float32.
+static constexpr double kCorrectF32 = 3e-12;
 __device__ void correct_rows_f32(const float* __restrict__ sUf, double* __restrict__ P, int b, int g, int ib0,
                                  int ib_end, int step, float* __restrict__ Pf) {
   const int rl = threadIdx.x / g, d = threadIdx.x - rl * g;
@@ -1336,7 +1339,7 @@ __global__ void __launch_bounds__(ORTH_T, 2) k_orth_coop(OrthCoopArgs a) {
       if (blockIdx.x == 0 && a.counters && threadIdx.x == 0)
         atomicMax(&a.counters[3], (unsigned long long)__double_as_longlong(defect));
       if (second && a.Tcol && a.nq > 0) compose_coefs(a.G1, a.G2, sR1, K, B, a.Tcol, a.ldT);
-      if (defect <= 1e-9) {
+      if (defect <= kCorrectF32) {
         float* sUf = reinterpret_cast<float*>(sC);
         for (int t = threadIdx.x; t < B * B; t += blockDim.x) sUf[t] = (float)sU[t];
         __syncthreads();
