@@ -133,7 +133,7 @@ typedef struct svt_options {
   int orth_tf32;          /* accepted and without effect: the coefficients of every Gram-Schmidt pass of the cooperative
                              orthonormalisation have float64 accuracy at the speed the split-TF32 products
                              this selected had */
-  int jacobi_cluster;     /* projected SVD: 0 (default) a thread-block cluster of 8 CTAs where the device
+  int jacobi_cluster;     /* FP64 projected SVD: 0 (default) a thread-block cluster of 8 CTAs where the device
                              allows it (the dense products, right vectors and residual estimates spread over
                              the cluster), else one CTA; 1: always one CTA (the same arithmetic but for the
                              grouping of sums) */

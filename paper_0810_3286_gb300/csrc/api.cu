@@ -633,7 +633,8 @@ static svt_status cycle_end(svt_ctx* c, int b, int J, int nk, bool copy_out) {
   const int nvec = std::max(1, nk) * b;
   l += prof_launch(c, SVT_PROF_JACOBI, 24.0 * K * K, [&] {
     return launch_small_svd(c->T, kKMax, K, c->Rkeep, b, nvec, c->theta, c->Xl, c->Wr, c->res, tol_j,
-                            c->prec != SVT_FP64, 60, c->err, c->dcount, c->gpart, c->st, c->opt.jacobi_cluster);
+                            c->prec != SVT_FP64, 60, c->err, c->dcount, c->gpart, c->st,
+                            c->prec == SVT_FP64 ? c->opt.jacobi_cluster : 0);
   });
   TRY(launched(c, l));
   if (!copy_out) return SVT_OK;
@@ -1010,7 +1011,8 @@ static svt_status shrink_randomized(svt_ctx* c, double tau, int s_init, int* r_o
     const double tol_j = c->prec == SVT_FP64 ? std::max(1e-15, 2.0 * l * 1.1102230246251565e-16) : 1e-9;
     int lj = prof_launch(c, SVT_PROF_JACOBI, 24.0 * l * l, [&] {
       return launch_small_svd(c->T, kKMax, l, nullptr, l, l, c->theta, c->Xl, c->Wr, c->res, tol_j,
-                              c->prec != SVT_FP64, 60, c->err, c->dcount, c->gpart, c->st, c->opt.jacobi_cluster);
+                              c->prec != SVT_FP64, 60, c->err, c->dcount, c->gpart, c->st,
+                            c->prec == SVT_FP64 ? c->opt.jacobi_cluster : 0);
     });
     TRY(launched(c, lj));
     CU(c, cudaMemcpyAsync(c->h_pin, c->theta, sizeof(double) * l, cudaMemcpyDeviceToHost, c->st));
