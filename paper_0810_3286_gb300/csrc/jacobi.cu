@@ -12,7 +12,8 @@
 //   2. k_psvd_refine: W back to orthonormality (float64 by one first-order step), then a first-order perturbation
 //      step on the leading nv columns, repeated until its own residual estimate meets the tolerance:
 //      S = W^T (T^T T) W[:, :nv], Theta_ji = the Jacobi angle of (S_ji, lambda_i, lambda_j), W <- W exp(Theta).  Everything
-//      is a matrix product; each step squares the error.  theta_i = ||T w_i||, x_i = T w_i / theta_i.
+//      is a matrix product; each step squares the error (as in Ogita and Aishima's refinement of eigenvectors).  theta_i =
+//      ||T w_i||, x_i = T w_i / theta_i.
 // Measured (GB300, one call, random block-bidiagonal T; before: float32 one-sided sweeps with accumulated rotations and
 // one float64 one-sided sweep, in CTA 0): K = 48, nv = 16: 533 -> 115 us (50 us sweeps, 65 us refinement); K = 72, nv = 24:
 // 1350 -> 281; K = 96, nv = 32: 3515 -> 490; K = 128, nv = 64: 9600 -> 1120 us; |T^T X - W theta| / sigma_1 from 1e-10 .. 1.6e-9 to

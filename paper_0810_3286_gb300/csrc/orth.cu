@@ -6,10 +6,10 @@
 // root ~650), so the sequence avoids long float64 dependency chains on a single SM:
 //   1. C1 = Q^T P                      (Gram, all SMs)
 //   2. P <- P - Q C1, [C2; A] = [Q, P]^T P   (one fused kernel: update + Gram of the same rows)
-//      R1 = chol(A)                    (four warps; reciprocal square root of each pivot seeded from
-//                                       its bits through a float32 rsqrt, one float64 Newton step;
+//      R1 = chol(A)                    (four warps; root-free, one reciprocal a pivot, seeded from its
+//                                       bits through a float32 reciprocal, one float64 Newton step;
 //                                       columns that lost all but 1e-12 of their norm to the
-//                                       projections are deflated to zero)
+//                                       projections are deflated)
 //   (the Grams and the projections of the cooperative kernel are digit products on the tensor cores, with the accuracy of
 //   float64 sums; those of the launch sequence are float64 instructions)
 //   3. P <- (P - Q C2) R1^-1, E = P^T P - I  (fused; per-row forward substitution, no inverse)
@@ -95,15 +95,17 @@ __device__ __forceinline__ void upper_ij(int t, int b, int& i, int& j) {
 
 // Partial Gram of rows [r0, r1) into partial[blockIdx.x * E ...), E = gram_entries(nq, b, first).
 // Called by all threads.
+// EPT: entries per thread, at least E / ORTH_T.
+template <int EPT = GRAM_EPT>
 __device__ void gram_chunk(const double* __restrict__ Q, long long q_stride, int nq, const double* __restrict__ P,
                            int b, int r0, int r1, double* __restrict__ partial, bool first) {
   __shared__ double tile[GRAM_SUB][GRAM_MAXW];
   const int W = (nq + 1) * b;
   const int E = gram_entries(nq, b, first);
   const int EQ = nq * b * b;
-  double acc[GRAM_EPT];
+  double acc[EPT];
 #pragma unroll
-  for (int k = 0; k < GRAM_EPT; ++k) acc[k] = 0.0;
+  for (int k = 0; k < EPT; ++k) acc[k] = 0.0;
   for (int rs = r0; rs < r1; rs += GRAM_SUB) {
     const int nr = min(GRAM_SUB, r1 - rs);
     for (int t = threadIdx.x; t < GRAM_SUB * W; t += blockDim.x) {
@@ -118,7 +120,7 @@ __device__ void gram_chunk(const double* __restrict__ Q, long long q_stride, int
     }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < GRAM_EPT; ++k) {
+    for (int k = 0; k < EPT; ++k) {
       int e = threadIdx.x + k * ORTH_T;
       if (e < E) {
         int c, d;
@@ -140,7 +142,7 @@ __device__ void gram_chunk(const double* __restrict__ Q, long long q_stride, int
     __syncthreads();
   }
 #pragma unroll
-  for (int k = 0; k < GRAM_EPT; ++k) {
+  for (int k = 0; k < EPT; ++k) {
     int e = threadIdx.x + k * ORTH_T;
     if (e < E) partial[(long long)blockIdx.x * E + e] = acc[k];
   }
@@ -646,7 +648,9 @@ int launch_correct(const double* G3, const double* R1, double* Tdiag, int ldT, d
 // v 2^(E - 62), |v| <= 2^62, and v splits into eight balanced base-256 digits, v = sum_k d_k 256^(7 - k), |d_k| <= 128,
 // each exact in float16.  Products of digits are at most 2^14, so sums over up to 128 terms of the (at most eight) pairs
 // with i + j = s stay within 2^24: the float32 accumulators are exact.  The pairs with i + j <= 7 (36 MMAs for a 16 x 8 x 16 step)
-// give the product to 2^-62 of its scale; the eight sums are put together in integers and rounded once.
+// are added up exactly, the eight sums put together in integers and rounded once.  What they leave out of a product is
+// below 2^-59 of its scale (seven pairs with i + j = 8 of up to 2^14 each), typically 2^-62.  (Splitting into exactly
+// representable slices for error-free products is the method of Ozaki, Ogita, Oishi and Rump.)
 // The exponents E are those of the CTA's rows: one for all of Q, one per column of P and of C.  (Seven digits lose more than
 // float64 sums do where rows differ by 10^4 and more in size: the orthogonality of such blocks went from 5e-16 to 3e-15.)
 // A fragment's elements are loaded (L1 holds the chunk) and split by the lane that needs them: no staging, no barriers.
@@ -1025,10 +1029,14 @@ __device__ void reduce_entries_ep(const double* __restrict__ partial, int nblk, 
     }
   }
 }
+// FEW: 8 columns, fewer entries than warps on large grids: fewer entries a warp and so one round of loads (n = 2753: 46.9 -> 45.4
+// us a block).
+template <bool FEW>
 __device__ __forceinline__ void reduce_entries(const double* __restrict__ partial, int nblk, int E,
                                                double* __restrict__ G, const double* Gprev, double* __restrict__ Tcol,
                                                int ldT, int ncoef, int b, unsigned int* err) {
-  if (nblk <= 128) reduce_entries_ep<4>(partial, nblk, E, G, Gprev, Tcol, ldT, ncoef, b, err);
+  if (FEW && nblk > 128) reduce_entries_ep<1>(partial, nblk, E, G, Gprev, Tcol, ldT, ncoef, b, err);
+  else if (nblk <= (FEW ? 64 : 128)) reduce_entries_ep<4>(partial, nblk, E, G, Gprev, Tcol, ldT, ncoef, b, err);
   else reduce_entries_ep<2>(partial, nblk, E, G, Gprev, Tcol, ldT, ncoef, b, err);
 }
 
@@ -1092,7 +1100,6 @@ struct OrthCoopArgs {
   const double* Q;            // nq blocks of rows x b, q_stride apart
   long long q_stride;
   int nq, n, g, rpc;          // rpc: rows per CTA
-  int fma;                    // float64 instructions instead of digit products (b = 8, small n)
   double *partial, *G1, *G2, *G3;
   long long part_half;        // doubles of one of the two sets of partials (0: one set)
   double *Tcol, *Tdiag;       // coefficient outputs (may be NULL), leading dimension ldT
@@ -1132,7 +1139,10 @@ __device__ void load_U_defect(const double* __restrict__ sG, int b, double* __re
   if ((threadIdx.x & 31) == 0) atomicMax(defect, mx);
 }
 
-template <int B>
+// FMA: float64 instructions instead of digit products (B = 8), a kernel of its own with no more code than it runs: every phase
+// runs once a launch, and fetching its instructions takes as long as running them.  In one kernel with the digit products and
+// with 20 entries a thread in gram_chunk, the second Gram took 9000 cycles at n = 1000; a block 37 us, now 31 (n = 200: 32.5 -> 28).
+template <int B, bool FMA>
 __global__ void __launch_bounds__(ORTH_T, 2) k_orth_coop(OrthCoopArgs a) {
   extern __shared__ double sm_orth[];
   double* sC = sm_orth;                 // K x B coefficients (C1, then C2)
@@ -1158,8 +1168,8 @@ __global__ void __launch_bounds__(ORTH_T, 2) k_orth_coop(OrthCoopArgs a) {
   if (threadIdx.x == 0) s_mq = s_def[0] = s_def[1] = 0;
   if (threadIdx.x < 2 * B) (&s_mp[0][0])[threadIdx.x] = 0;
   __syncthreads();
-  const bool digits = B != 8 || !a.fma;
-  if (digits) dg_maxima<B>(a.Q, a.q_stride, a.nq, a.P, r0, r1, &s_mq, s_mp[0]);
+  constexpr bool digits = !FMA;
+  if constexpr (digits) dg_maxima<B>(a.Q, a.q_stride, a.nq, a.P, r0, r1, &s_mq, s_mp[0]);
   __syncthreads();
   const int eq = dg_exponent(s_mq);
   // exponents of P's columns from the maxima in s_mp[cur]; the other set is cleared for the next change of P
@@ -1175,23 +1185,16 @@ __global__ void __launch_bounds__(ORTH_T, 2) k_orth_coop(OrthCoopArgs a) {
   next_exponents();
   // Partial Gram [Q_0 .. Q_{nq-1}, P]^T P of the CTA's rows; P <- P - Q C from warp w0 on (bar as for dg_update)
   auto gram = [&](int nq, double* part, bool first) {
-    if constexpr (B == 8) {
-      if (a.fma) {
-        __syncthreads();
-        gram_chunk(a.Q, a.q_stride, nq, a.P, B, r0, r1, part, first);
-        return;
-      }
+    if constexpr (FMA) {
+      __syncthreads();
+      gram_chunk<(GRAM_MAXW * B + ORTH_T - 1) / ORTH_T>(a.Q, a.q_stride, nq, a.P, B, r0, r1, part, first);
+    } else {
+      dg_gram<B>(a.Q, a.q_stride, nq, a.P, r0, r1, eq, s_ep, part, first, s_red);
     }
-    dg_gram<B>(a.Q, a.q_stride, nq, a.P, r0, r1, eq, s_ep, part, first, s_red);
   };
   auto project = [&](int w0, int bar) {
-    if constexpr (B == 8) {
-      if (a.fma) {
-        update_rows(0, a.Q, a.q_stride, a.nq, sC, nullptr, nullptr, a.P, B, a.g, r0, r1, nullptr, 32 * w0);
-        return;
-      }
-    }
-    dg_update<B>(a.Q, a.q_stride, a.nq, sC, s_ec, eq, a.P, r0, r1, s_mp[cur], w0, nw - w0, s_red, bar);
+    if constexpr (FMA) update_rows(0, a.Q, a.q_stride, a.nq, sC, nullptr, nullptr, a.P, B, a.g, r0, r1, nullptr, 32 * w0);
+    else dg_update<B>(a.Q, a.q_stride, a.nq, sC, s_ec, eq, a.P, r0, r1, s_mp[cur], w0, nw - w0, s_red, bar);
   };
   // Where every CTA adds up a Gram for itself, one may still read its partials while another writes the next Gram's: two sets
   // in turn.  (Else a barrier follows the sums, and the sets are the same.)
@@ -1206,7 +1209,7 @@ __global__ void __launch_bounds__(ORTH_T, 2) k_orth_coop(OrthCoopArgs a) {
     if (nq == 0 && nb <= OC_SETS_GRID) {   // (with coefficients the CTAs' reads take longer than the barrier: 16000 cycles at n = 1000)
       reduce_all(part, nb, E, G, Gprev, Tcol, a.ldT, nc, B, sC, sTail, err);
     } else {
-      reduce_entries(part, nb, E, G, Gprev, Tcol, a.ldT, nc, B, err);
+      reduce_entries<FMA>(part, nb, E, G, Gprev, Tcol, a.ldT, nc, B, err);
       if (!svt_grid_barrier(a.bar, a.err, a.spin_limit)) return false;
       for (int e = threadIdx.x; e < E; e += ORTH_T) {
         const double v = __ldcg(G + e);
@@ -1228,14 +1231,14 @@ __global__ void __launch_bounds__(ORTH_T, 2) k_orth_coop(OrthCoopArgs a) {
       gram(a.nq, partial, true);
       if (!gram_sums(a.nq, true, a.G1, nullptr, nullptr, sRef, a.err)) return;
       // P <- P - Q C1; [C2; A] = [Q, P]^T P; coefficients C1 + C2 -> Tcol (first pass)
-      if (digits) dg_col_exponents<B>(sC, K, s_ec, 0, nw);
+      if constexpr (digits) dg_col_exponents<B>(sC, K, s_ec, 0, nw);
       __syncthreads();
       project(0, 3);
       __syncthreads();
       next_exponents();
       gram(a.nq, partial, false);
       if (!gram_sums(a.nq, false, a.G2, a.G1, pass == 0 ? a.Tcol : nullptr, sTail, nullptr)) return;
-      if (digits) dg_col_exponents<B>(sC, K, s_ec, 0, nw);
+      if constexpr (digits) dg_col_exponents<B>(sC, K, s_ec, 0, nw);
       __syncthreads();
     } else {
       gram(0, partial, false);
@@ -1285,7 +1288,7 @@ __global__ void __launch_bounds__(ORTH_T, 2) k_orth_coop(OrthCoopArgs a) {
       by_row = r1 - r0 >= 64;
       if (by_row) solve_rows<B>(sR2, sD, a.P, r0, r1, s_mp[cur]);
     }
-    if (!by_row) update_rows(1, nullptr, 0, 0, nullptr, sR2, sD, a.P, B, a.g, r0, r1, s_mp[cur]);
+    if (!by_row) update_rows(1, nullptr, 0, 0, nullptr, sR2, sD, a.P, B, a.g, r0, r1, digits ? s_mp[cur] : nullptr);
     if (ndef > 0) {
       __syncthreads();   // the substitution above wrote these rows
       // the seed comes from R, identical in every CTA and different from block to block
@@ -1377,16 +1380,16 @@ __global__ void __launch_bounds__(ORTH_T, 2) k_orth_coop(OrthCoopArgs a) {
   }
 }
 
-template <int B>
+template <int B, bool FMA>
 static bool orth_coop_attr() {
-  return cudaFuncSetAttribute(k_orth_coop<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(k_orth_coop<B, FMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)orth_coop_smem(B)) == cudaSuccess;
 }
 
-template <int B>
+template <int B, bool FMA>
 static int orth_coop_blocks_per_sm() {
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_orth_coop<B>, ORTH_T, orth_coop_smem(B)) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_orth_coop<B, FMA>, ORTH_T, orth_coop_smem(B)) != cudaSuccess)
     return 0;
   return nb;
 }
@@ -1405,12 +1408,14 @@ int orth_coop_init() {
       (void)cudaGetLastError();
       return;
     }
-    if (!orth_coop_attr<8>() || !orth_coop_attr<16>() || !orth_coop_attr<24>() || !orth_coop_attr<32>()) {
+    if (!orth_coop_attr<8, true>() || !orth_coop_attr<8, false>() || !orth_coop_attr<16, false>() ||
+        !orth_coop_attr<24, false>() || !orth_coop_attr<32, false>()) {
       (void)cudaGetLastError();
       return;
     }
-    int bps = std::min(std::min(orth_coop_blocks_per_sm<8>(), orth_coop_blocks_per_sm<16>()),
-                       std::min(orth_coop_blocks_per_sm<24>(), orth_coop_blocks_per_sm<32>()));
+    int bps = std::min({orth_coop_blocks_per_sm<8, true>(), orth_coop_blocks_per_sm<8, false>(),
+                        orth_coop_blocks_per_sm<16, false>(), orth_coop_blocks_per_sm<24, false>(),
+                        orth_coop_blocks_per_sm<32, false>()});
     bps = std::min(bps, 2);
     grid = bps * sms;
   });
@@ -1424,13 +1429,13 @@ int launch_orth_coop(double* P, const double* Q, long long q_stride, int nq, int
   const int gmax = std::min(orth_coop_init(), max_grid);
   if (gmax <= 0 || n <= 0) return 0;
   // At least 16 rows per CTA (a step of the digit products) and at most gmax CTAs.  A block of 8 columns of a small problem
-  // leaves most warps without a tile, and float64 instructions on chunks of 8 rows take less (n = 200, nq = 2: 29 us
-  // against 36); n = 200, b = 16 takes 47 us either way.
-  const bool fma = b == 8 && n <= 8 * gmax;
+  // leaves most warps without a tile; float64 instructions on chunks of 8 and more rows take less (us, nq = 2 or so: n = 2753
+  // 42.9 against 45.4, 7000 49.7 against 52.5, 10000 61.8 against 55.5); n = 200, b = 16 takes 47 us either way.
+  const bool fma = b == 8 && n <= 24 * gmax;
   const int rpc = std::max(fma ? 8 : 16, (n + gmax - 1) / gmax);
   const int grid = (n + rpc - 1) / rpc;
   OrthCoopArgs a;
-  a.P = P; a.Q = Q; a.q_stride = q_stride; a.nq = nq; a.n = n; a.g = row_group(b); a.rpc = rpc; a.fma = fma ? 1 : 0;
+  a.P = P; a.Q = Q; a.q_stride = q_stride; a.nq = nq; a.n = n; a.g = row_group(b); a.rpc = rpc;
   a.partial = partial; a.part_half = grid <= OC_SETS_GRID ? (long long)grid * gram_entries(nq, b, false) : 0; a.G1 = G1; a.G2 = G2; a.G3 = G3;
   a.Tcol = Tcol; a.Tdiag = Tdiag; a.ldT = ldT; a.Pf = Pf;
   a.counters = counters; a.err = err; a.bar = static_cast<unsigned int*>(bar); a.twoc = twoc;
@@ -1448,10 +1453,10 @@ int launch_orth_coop(double* P, const double* Q, long long q_stride, int nq, int
   cfg.numAttrs = 1;
   cudaError_t e;
   switch (b) {
-    case 8: e = cudaLaunchKernelEx(&cfg, k_orth_coop<8>, a); break;
-    case 16: e = cudaLaunchKernelEx(&cfg, k_orth_coop<16>, a); break;
-    case 24: e = cudaLaunchKernelEx(&cfg, k_orth_coop<24>, a); break;
-    case 32: e = cudaLaunchKernelEx(&cfg, k_orth_coop<32>, a); break;
+    case 8: e = fma ? cudaLaunchKernelEx(&cfg, k_orth_coop<8, true>, a) : cudaLaunchKernelEx(&cfg, k_orth_coop<8, false>, a); break;
+    case 16: e = cudaLaunchKernelEx(&cfg, k_orth_coop<16, false>, a); break;
+    case 24: e = cudaLaunchKernelEx(&cfg, k_orth_coop<24, false>, a); break;
+    case 32: e = cudaLaunchKernelEx(&cfg, k_orth_coop<32, false>, a); break;
     default: return 0;
   }
   return e == cudaSuccess ? 1 : 0;
