@@ -140,7 +140,8 @@ __device__ __forceinline__ void spmm_pieces(const int32_t* __restrict__ idx, con
                                             const XT* __restrict__ X, int b, int G, int piece, int lo, int hi,
                                             double* row, double (&w)[CPL], int& col, int& n) {
   const int np = (hi - lo + piece / 2) / piece;
-  const int len = np > 1 ? (hi - lo + np - 1) / np : hi - lo;
+  const int group = 4 * (32 / G);                  // entries of an unrolled step: only the last piece has a ragged end
+  const int len = np > 1 ? ((hi - lo + np - 1) / np + group - 1) / group * group : hi - lo;
   for (int p = lo;;) {
     const int q = min(hi, p + len);
     spmm_sum<VT, XT, AT, CPL>(idx, val, X, b, G, p, q, w, col, n);
@@ -157,10 +158,10 @@ __device__ __forceinline__ void spmm_pieces(const int32_t* __restrict__ idx, con
 
 // Tile `tile` of the `tiles` of one product, by the whole CTA: the segments tile + k tiles, k < (SPMM_T / 32) / WPR, WPR warps
 // each.  Segments of more than `longw` entries a warp are shared by all its warps; neighbours, which tend to be long together
-// (rows in the order of their popularity), belong to different tiles.  Measured (us, float64, b = 16): 10000 segments of 120 of
+// (rows in the order of their popularity), belong to different tiles.  PIECES: with the loop over pieces.  Measured (us, float64, b = 16): 10000 segments of 120 of
 // which the last eight have 1000, neighbours in one tile / in different ones: 110 / 57 (two segments a CTA with four warps
 // each: 73).
-template <typename VT, typename XT, typename AT>
+template <typename VT, typename XT, typename AT, bool PIECES>
 __device__ __forceinline__ void spmm_tile(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                                           const VT* __restrict__ val, const XT* __restrict__ X,
                                           double* __restrict__ Out, int n_out, int b, int G, int WPR, int piece,
@@ -174,7 +175,10 @@ __device__ __forceinline__ void spmm_tile(const int32_t* __restrict__ ptr, const
     const int lo = min(e, a + wp * chunk);
     double w[CPL];
     int col, n;
-    spmm_pieces<VT, XT, AT, CPL>(idx, val, X, b, G, piece, lo, min(e, lo + chunk), part[warp], w, col, n);
+    if constexpr (PIECES)
+      spmm_pieces<VT, XT, AT, CPL>(idx, val, X, b, G, piece, lo, min(e, lo + chunk), part[warp], w, col, n);
+    else
+      spmm_sum<VT, XT, AT, CPL>(idx, val, X, b, G, lo, min(e, lo + chunk), w, col, n);
     spmm_store<CPL>((share > 1 ? part[warp] : out) + col, w, n);
   };
   // the sums of `share` warps from warp w0 on, by the threads t0, t0 + nt, ...
@@ -208,28 +212,28 @@ __device__ __forceinline__ void spmm_tile(const int32_t* __restrict__ ptr, const
   if (WPR > 1 || any) __syncthreads();
 }
 
-template <typename VT, typename XT, typename AT>
+template <typename VT, typename XT, typename AT, bool PIECES>
 __global__ void __launch_bounds__(SPMM_T, 5)
 k_spmm(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx, const VT* __restrict__ val,
        const XT* __restrict__ X, double* __restrict__ Out, int n_out, int b, int G, int WPR, int piece, int longw) {
   const int segs_per_block = (SPMM_T / 32) / WPR;
   const int tiles = (n_out + segs_per_block - 1) / segs_per_block;
   for (int t = blockIdx.x; t < tiles; t += gridDim.x)
-    spmm_tile<VT, XT, AT>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, longw, t, tiles);
+    spmm_tile<VT, XT, AT, PIECES>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, longw, t, tiles);
 }
 
 // Ragged persistent form over a job list (batched engine): the tiles of all listed products form
 // one index space (job k owns tiles tile0 .. tile0 + ceil(n_out / segments per tile) - 1); each CTA
 // takes tiles grid-stride and finds the job of a tile by a scan of the (at most kBatchMaxJobs)
 // offsets.  Every segment is computed exactly as k_spmm computes it with the same G and WPR.
-template <typename VT, typename XT, typename AT>
+template <typename VT, typename XT, typename AT, bool PIECES>
 __global__ void __launch_bounds__(SPMM_T) k_spmm_jobs(const __grid_constant__ SpmmJobTable tab) {
   for (int t = blockIdx.x; t < tab.tiles; t += gridDim.x) {
     int k = 0;
     while (k + 1 < tab.n && tab.job[k + 1].tile0 <= t) ++k;
     const SpmmJobDev& J = tab.job[k];
     const int segs_per_block = (SPMM_T / 32) / J.WPR;
-    spmm_tile<VT, XT, AT>(J.ptr, J.idx, static_cast<const VT*>(J.val), static_cast<const XT*>(J.X), J.Out, J.n_out,
+    spmm_tile<VT, XT, AT, PIECES>(J.ptr, J.idx, static_cast<const VT*>(J.val), static_cast<const XT*>(J.X), J.Out, J.n_out,
                           J.b, J.G, J.WPR, J.piece, J.longw, t - J.tile0, (J.n_out + segs_per_block - 1) / segs_per_block);
   }
 }
@@ -248,19 +252,22 @@ static void spmm_shape(int CPL, bool f32, int b, long long nnz, int n_out, int w
   // 1000 of 120 float64 16.6 / 13.8 / 16.  Where a warp has over 48 steps to go, more and shorter ones even out the last wave
   // and cost less, up to 16384 (limit of 4096 / 16384): 2797 segments of 348, b = 48, float64 113 / 109; 5000 of 300, b = 32, 105 /
   // 89; 5000 of 250, b = 16, 51 / 47; 15000 of 300, b = 32, 253 / 242.
+  const int ngrp = 32 / G;
   const double mean_len = nnz > 0 ? (double)nnz / n_out : 0.0;
   int WPR = 1;
-  while (WPR < 8 && mean_len / WPR > 8.0 * (32 / G) &&
-         (long long)n_out * WPR < (mean_len / WPR > 48.0 * (32 / G) ? 16384 : 4096))
+  while (WPR < 8 && mean_len / WPR > 8.0 * ngrp &&
+         ((long long)n_out * WPR < (mean_len / WPR > 48.0 * ngrp ? 16384 : 4096) || (CPL == 4 && mean_len / WPR > 32.0 * ngrp)))
     WPR <<= 1;
   if (wpr_override == 1 || wpr_override == 2 || wpr_override == 4 || wpr_override == 8) WPR = wpr_override;
-  // Pieces: a lane's two sums take at most 16 entries each (times 3/2 where a length is no multiple of the piece), and no more
-  // than half of what `shares` warps would leave a lane of a mean segment.  In float64, with 2^-53 an addition, no more than
-  // all of that, and never less than half.  Measured, whole segments -> pieces (error of both products and the update against
-  // 64 bits): 24000 x 20000, 520 entries a segment, b = 48: float32 2.9e-7 -> 8.7e-8 (the three calls 3.33 -> 3.51 ms), float64
-  // 8.7e-16 -> 8.2e-16 (3.48 -> 3.53 ms); 9000 x 11000, 267, b = 32: float32 1.5e-7 -> 8.8e-8, float64 6.1e-16 -> 5.8e-16.  Mean
-  // segments of 120 entries at b = 16 are one piece.
-  const int ngrp = 32 / G;
+  // Pieces, where a mean segment needs several: a lane's two sums take at most 16 entries each (times 3/2 where a length is no
+  // multiple of the piece), and no more than half of what `shares` warps would leave a lane of a mean segment.  In float64, with
+  // 2^-53 an addition, no more than all of that, and never less than half.  Measured, whole segments -> pieces (error of both
+  // products and the update against 64 bits): 24000 x 20000, 520 entries a segment, b = 48: float32 2.9e-7 -> 8.7e-8 (the three
+  // calls 3.33 -> 3.51 ms), float64 8.7e-16 -> 8.2e-16 (3.48 -> 3.53 ms); 9000 x 11000, 267, b = 32: float32 1.5e-7 -> 8.8e-8, float64
+  // 6.1e-16 -> 5.8e-16.
+  // Elsewhere, and for float32 blocks (CPL = 4, the products of the solves), the kernel without that loop, which costs it 9 to 28 %
+  // (float32, 30000 segments of 120, b = 16, 34 -> 37 us; 4219 of 111, b = 24, 12.4 -> 16.2): a warp takes at most 48 steps (float32;
+  // chains of 24 additions) or 96 of a segment, and float32 blocks have more warps a segment from 32 steps on.
   int shares = 1;
   while (shares < 8 && mean_len / shares > 8.0 * ngrp) shares <<= 1;
   int piece = 32 * ngrp;
@@ -268,12 +275,14 @@ static void spmm_shape(int CPL, bool f32, int b, long long nnz, int n_out, int w
     const int half = 2 * (int)std::ceil(mean_len / shares);
     piece = f32 ? std::min(piece, half) : std::max(std::min(piece, 2 * half), half);
   }
+  if (CPL == 4 || mean_len / WPR < 1.5 * piece) piece = 0;
   *G_out = G;
   *WPR_out = WPR;
   *piece_out = piece;
   // A warp takes three mean segments (or 64 steps) at most.  Measured (us, float64, b = 16, factors 8 / 4 / 3 / 2): 10000 segments
   // of power-law lengths (exponent 2, mean 120) 96 / 84 / 79 / 79; 3000 of 120 with two of 1000 43 / 29 / 29 / 29.
   *longw_out = std::max((int)std::min(3.0 * std::ceil(mean_len / WPR), 134217728.0), 64 * ngrp);
+  if (piece == 0) *longw_out = std::min(*longw_out, (f32 ? 48 : 96) * ngrp);
 }
 
 template <typename VT, typename XT, typename AT>
@@ -284,7 +293,10 @@ static void spmm_launch(const int32_t* ptr, const int32_t* idx, const VT* val, c
   spmm_shape(CPL, sizeof(AT) == 4, b, nnz, n_out, 0, &G, &WPR, &piece, &longw);
   const int segs_per_block = (SPMM_T / 32) / WPR;
   int blocks = (int)svt_min_ll(svt_ceil_div(n_out, segs_per_block), 152LL * 16);
-  k_spmm<VT, XT, AT><<<blocks, SPMM_T, 0, st>>>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, longw);
+  if (sizeof(XT) == 4 || piece == 0)
+    k_spmm<VT, XT, AT, false><<<blocks, SPMM_T, 0, st>>>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, longw);
+  else
+    k_spmm<VT, XT, AT, sizeof(XT) == 8><<<blocks, SPMM_T, 0, st>>>(ptr, idx, val, X, Out, n_out, b, G, WPR, piece, longw);
 }
 
 // One launch for the products of a job list: precision as launch_spmm (0 float64, 1 float32 values
@@ -294,6 +306,7 @@ int launch_spmm_jobs(int precision, const SpmmJob* jobs, int n, int grid, cudaSt
   SpmmJobTable tab{};
   tab.n = 0;
   int tiles = 0;
+  bool pieces = false;
   const int CPL = precision == 0 ? XRow<double>::CPL : XRow<float>::CPL;
   for (int k = 0; k < n; ++k) {
     const SpmmJob& J = jobs[k];
@@ -303,15 +316,17 @@ int launch_spmm_jobs(int precision, const SpmmJob* jobs, int n, int grid, cudaSt
     d.X = precision == 0 ? static_cast<const void*>(J.X) : static_cast<const void*>(J.Xf);
     if (!d.X) return 0;
     spmm_shape(CPL, precision != 0, J.b, J.nnz, J.n_out, J.wpr, &d.G, &d.WPR, &d.piece, &d.longw);
+    pieces = pieces || d.piece > 0;
     d.tile0 = tiles;
     tiles += (J.n_out + (SPMM_T / 32) / d.WPR - 1) / ((SPMM_T / 32) / d.WPR);
   }
   if (tab.n == 0) return 0;
   tab.tiles = tiles;
   const int blocks = std::max(1, std::min(tiles, grid > 0 ? grid : 152 * 16));
-  if (precision == 2) k_spmm_jobs<__nv_bfloat16, float, float><<<blocks, SPMM_T, 0, st>>>(tab);
-  else if (precision == 0) k_spmm_jobs<double, double, double><<<blocks, SPMM_T, 0, st>>>(tab);
-  else k_spmm_jobs<float, float, float><<<blocks, SPMM_T, 0, st>>>(tab);
+  if (precision == 2) k_spmm_jobs<__nv_bfloat16, float, float, false><<<blocks, SPMM_T, 0, st>>>(tab);
+  else if (precision == 0 && pieces) k_spmm_jobs<double, double, double, true><<<blocks, SPMM_T, 0, st>>>(tab);
+  else if (precision == 0) k_spmm_jobs<double, double, double, false><<<blocks, SPMM_T, 0, st>>>(tab);
+  else k_spmm_jobs<float, float, float, false><<<blocks, SPMM_T, 0, st>>>(tab);
   return 1;
 }
 
