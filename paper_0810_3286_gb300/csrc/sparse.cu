@@ -212,8 +212,10 @@ __device__ __forceinline__ void spmm_tile(const int32_t* __restrict__ ptr, const
   if (WPR > 1 || any) __syncthreads();
 }
 
+// Resident CTAs an SM: five (48 registers); eight for float32 sums of float64 blocks without pieces, whose products of few
+// long segments are one wave with them (1033 segments of 340 at b = 46, eight warps each: 53.2 -> 50.3 us).
 template <typename VT, typename XT, typename AT, bool PIECES>
-__global__ void __launch_bounds__(SPMM_T, 5)
+__global__ void __launch_bounds__(SPMM_T, !PIECES && sizeof(XT) == 8 && sizeof(AT) == 4 ? 8 : 5)
 k_spmm(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx, const VT* __restrict__ val,
        const XT* __restrict__ X, double* __restrict__ Out, int n_out, int b, int G, int WPR, int piece, int longw) {
   const int segs_per_block = (SPMM_T / 32) / WPR;
